@@ -556,89 +556,267 @@ __global__ void conf_features_kernel(const float *__restrict__ depth, Intr in, f
     for (int k = 0; k < NF; ++k) feat[(size_t)s * NF + k] = x[k];
 }
 
-// scratch per sample: h1 (bf16-rounded), h2, d2, d1 (64 each), dout
-constexpr int kSH1 = 0, kSH2 = 64, kSD2 = 128, kSD1 = 192, kSDO = 256, kSRow = ITM_MLP_SCRATCH_PER_SAMPLE;
+// Training step (mlp_step_kernel, then mlp_reduce_kernel).  A CTA takes 64
+// samples at a time through the whole step in shared memory: forward, loss,
+// both deltas, and the tile's share of every parameter's gradient, which it
+// keeps in registers over its tiles (a 4 x 4 patch of W2's gradient and one
+// of W1's per thread) and writes as one row of partial sums at its end.  The
+// reduction adds the rows in a fixed order, so gradient and loss do not
+// depend on scheduling.  The five products are register-tiled (4 x 4 outputs
+// per thread, operands as float4 from shared memory); each output is one
+// chain of FMAs in the order bias, k = 0, 1, ..., so a forward value and its
+// bfloat16 rounding are those of a plain loop.
+//
+// Bound: FP32 issue within a CTA (19 k FMAs per sample, 1.2 M per tile); at
+// the training's 8192 samples 128 CTAs on 152 SMs run one tile each.  Before,
+// one thread took a whole sample (64 CTAs, activations in global memory) and
+// one thread per parameter then walked all samples: 53 + 377 us for 8192
+// samples; now 16 + 2.5 us (22 us before the weights and the tile were loaded
+// by whole counts of loads issued together).  64 samples per tile: the
+// largest that leaves one tile per SM at 8192 samples, and the rows of
+// partial sums then fit the caller's scratch for every sample count (below).
+constexpr int kTS = 64, kStepThreads = 256;
+constexpr int kXS = NF;      // row stride of x and W1 (floats): 8 rows of 16 B on distinct banks
+constexpr int kHS = NH + 4;  // row stride of the 64-wide tiles, likewise
+static_assert(NF % 4 == 0 && NF == 52 && NH == 64 && kTS == 64, "float4 rows without bank conflicts, 16 x 16 threads");
+constexpr int kPartial = NP + 1;  // a row of partial sums: every parameter's gradient, the loss
+// rows (one per CTA) fit the scratch of kSRow floats per sample: two rows need
+// at least kTS + 1 samples, every further row kTS more; one row needs none
+constexpr int kSRow = ITM_MLP_SCRATCH_PER_SAMPLE;
+static_assert(2 * kPartial <= (kTS + 1) * kSRow && kPartial <= kTS * kSRow, "partial sums in the scratch");
 
-__global__ void __launch_bounds__(128) mlp_fwd_bwd_kernel(const float *__restrict__ P, const float *__restrict__ feat,
-                                                          const float *__restrict__ y, int n,
-                                                          float *__restrict__ scratch, float *__restrict__ loss)
+struct StepSmem {
+    float W1[NH * kXS], x[kTS * kXS];
+    float W2[NH * kHS], h1[kTS * kHS], h2[kTS * kHS], d2[kTS * kHS], d1[kTS * kHS];
+    float b1[NH], b2[NH], w3[NH], dout[kTS], loss[kTS];
+    float b3;
+};
+
+// acc[i][j] += sum over q < 4 of a[i].q b[j].q, in the order of q
+__device__ __forceinline__ void dot4x4(float (&acc)[4][4], const float4 (&a)[4], const float4 (&b)[4])
 {
-    __shared__ float sW1[NH * NF], sW2[NH * NH], sB1[NH], sB2[NH], sW3[NH], sB3;
-    __shared__ float sLoss[4];
-    for (int i = threadIdx.x; i < NH * NF; i += blockDim.x) sW1[i] = bf16r(P[P_W1 + i]);
-    for (int i = threadIdx.x; i < NH * NH; i += blockDim.x) sW2[i] = bf16r(P[P_W2 + i]);
-    for (int i = threadIdx.x; i < NH; i += blockDim.x) {
-        sB1[i] = P[P_B1 + i];
-        sB2[i] = P[P_B2 + i];
-        sW3[i] = P[P_W3 + i];
-    }
-    if (threadIdx.x == 0) sB3 = P[P_B3];
-    __syncthreads();
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    float l = 0.0f;
-    if (s < n) {
-        float *row = scratch + (size_t)s * kSRow;
-        float x[NF];
-        for (int k = 0; k < NF; ++k) x[k] = bf16r(feat[(size_t)s * NF + k]);
-        for (int m = 0; m < NH; ++m) {
-            float a = sB1[m];
-            for (int k = 0; k < NF; ++k) a = fmaf(sW1[m * NF + k], x[k], a);
-            row[kSH1 + m] = bf16r(fmaxf(a, 0.0f));  // as consumed by layer 2; 0 where the ReLU is off
-        }
-        float o = sB3;
-        for (int a = 0; a < NH; ++a) {
-            float acc = sB2[a];
-            for (int m = 0; m < NH; ++m) acc = fmaf(sW2[a * NH + m], row[kSH1 + m], acc);
-            const float h2 = fmaxf(acc, 0.0f);
-            row[kSH2 + a] = h2;
-            o = fmaf(sW3[a], h2, o);
-        }
-        const float t = y[s];
-        const float p = 1.0f / (1.0f + expf(-o));
-        l = fmaxf(o, 0.0f) - o * t + log1pf(expf(-fabsf(o)));
-        const float dout = (p - t) / (float)n;
-        row[kSDO] = dout;
-        for (int a = 0; a < NH; ++a) row[kSD2 + a] = row[kSH2 + a] > 0.0f ? dout * sW3[a] : 0.0f;
-        for (int m = 0; m < NH; ++m) {
-            float acc = 0.0f;
-            for (int a = 0; a < NH; ++a) acc = fmaf(sW2[a * NH + m], row[kSD2 + a], acc);
-            row[kSD1 + m] = row[kSH1 + m] > 0.0f ? acc : 0.0f;
-        }
-    }
-    // loss: warp sums, one atomic per CTA
-    for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(kFull, l, o);
-    if ((threadIdx.x & 31) == 0) sLoss[threadIdx.x >> 5] = l;
-    __syncthreads();
-    if (threadIdx.x == 0) atomicAdd(loss, (sLoss[0] + sLoss[1] + sLoss[2] + sLoss[3]) / (float)n);
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                acc[i][j] = fmaf(reinterpret_cast<const float *>(&b[j])[q], reinterpret_cast<const float *>(&a[i])[q],
+                                 acc[i][j]);
 }
 
-// one thread per parameter, summing its gradient over the batch
-__global__ void mlp_grad_kernel(const float *__restrict__ feat, const float *__restrict__ scratch, int n,
-                                float *__restrict__ grad)
+__device__ __forceinline__ float4 ld4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
+
+__global__ void __launch_bounds__(kStepThreads) mlp_step_kernel(const float *__restrict__ P,
+                                                                const float *__restrict__ feat,
+                                                                const float *__restrict__ y, int n,
+                                                                float *__restrict__ out, float *__restrict__ loss)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= NP) return;
-    float acc = 0.0f;
-    if (i < P_B1) {
-        const int m = i / NF, k = i % NF;
-        for (int s = 0; s < n; ++s) acc = fmaf(scratch[(size_t)s * kSRow + kSD1 + m], bf16r(feat[(size_t)s * NF + k]), acc);
-    } else if (i < P_W2) {
-        const int m = i - P_B1;
-        for (int s = 0; s < n; ++s) acc += scratch[(size_t)s * kSRow + kSD1 + m];
-    } else if (i < P_B2) {
-        const int a = (i - P_W2) / NH, m = (i - P_W2) % NH;
-        for (int s = 0; s < n; ++s)
-            acc = fmaf(scratch[(size_t)s * kSRow + kSD2 + a], scratch[(size_t)s * kSRow + kSH1 + m], acc);
-    } else if (i < P_W3) {
-        const int a = i - P_B2;
-        for (int s = 0; s < n; ++s) acc += scratch[(size_t)s * kSRow + kSD2 + a];
-    } else if (i < P_B3) {
-        const int a = i - P_W3;
-        for (int s = 0; s < n; ++s) acc = fmaf(scratch[(size_t)s * kSRow + kSDO], scratch[(size_t)s * kSRow + kSH2 + a], acc);
-    } else {
-        for (int s = 0; s < n; ++s) acc += scratch[(size_t)s * kSRow + kSDO];
+    extern __shared__ __align__(16) unsigned char step_smem[];
+    StepSmem &S = *reinterpret_cast<StepSmem *>(step_smem);
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    // whole counts of loads per thread, issued together: one trip to L2 each
+    static_assert(NH * NF % kStepThreads == 0 && NH * NH % kStepThreads == 0 && kTS * NF % kStepThreads == 0, "loads");
+#pragma unroll
+    for (int i = tid; i < NH * NF; i += kStepThreads) S.W1[i] = bf16r(__ldg(&P[P_W1 + i]));
+#pragma unroll
+    for (int i = tid; i < NH * NH; i += kStepThreads) S.W2[(i >> 6) * kHS + (i & 63)] = bf16r(__ldg(&P[P_W2 + i]));
+    if (tid < NH) {
+        S.b1[tid] = P[P_B1 + tid];
+        S.b2[tid] = P[P_B2 + tid];
+        S.w3[tid] = P[P_W3 + tid];
     }
-    grad[i] = acc;
+    if (tid == 0) S.b3 = P[P_B3];
+    float g1[4][4] = {}, g2[4][4] = {};  // W1: rows 4 ty + i, columns 4 tx + j (tx < 13); W2: rows 4 ty + i, columns 4 tx + j
+    float gv = 0.0f, gl = 0.0f;          // thread q * 64 + m: b1, b2, w3 (q = 0, 1, 2) of unit m; b3 and the loss
+    for (int s0 = blockIdx.x * kTS; s0 < n; s0 += gridDim.x * kTS) {
+        const int ns = min(kTS, n - s0);
+        __syncthreads();  // the previous tile is no longer read
+#pragma unroll
+        for (int i = tid; i < kTS * NF; i += kStepThreads)
+            S.x[i] = i < ns * NF ? bf16r(__ldg(&feat[(size_t)s0 * NF + i])) : 0.0f;
+        __syncthreads();
+        // h1 = relu(W1 x + b1), rounded as layer 2 consumes it: samples ty + 16 i, units tx + 16 j
+        {
+            float acc[4][4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[i][j] = S.b1[tx + 16 * j];
+#pragma unroll 1
+            for (int k = 0; k < NF; k += 4) {
+                float4 a[4], b[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) a[i] = ld4(&S.x[(ty + 16 * i) * kXS + k]);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) b[j] = ld4(&S.W1[(tx + 16 * j) * kXS + k]);
+                dot4x4(acc, a, b);
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    S.h1[(ty + 16 * i) * kHS + tx + 16 * j] = ty + 16 * i < ns ? bf16r(fmaxf(acc[i][j], 0.0f)) : 0.0f;
+        }
+        __syncthreads();
+        // h2 = relu(W2 h1 + b2)
+        {
+            float acc[4][4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[i][j] = S.b2[tx + 16 * j];
+#pragma unroll 2
+            for (int k = 0; k < NH; k += 4) {
+                float4 a[4], b[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) a[i] = ld4(&S.h1[(ty + 16 * i) * kHS + k]);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) b[j] = ld4(&S.W2[(tx + 16 * j) * kHS + k]);
+                dot4x4(acc, a, b);
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    S.h2[(ty + 16 * i) * kHS + tx + 16 * j] = ty + 16 * i < ns ? fmaxf(acc[i][j], 0.0f) : 0.0f;
+        }
+        __syncthreads();
+        // output, loss and its derivative, one thread per sample
+        if (tid < kTS) {
+            float l = 0.0f, d = 0.0f;
+            if (tid < ns) {
+                float o = S.b3;
+#pragma unroll
+                for (int a = 0; a < NH; a += 4) {
+                    const float4 h = ld4(&S.h2[tid * kHS + a]), w = ld4(&S.w3[a]);
+                    o = fmaf(w.w, h.w, fmaf(w.z, h.z, fmaf(w.y, h.y, fmaf(w.x, h.x, o))));
+                }
+                const float t = y[s0 + tid];
+                const float p = 1.0f / (1.0f + expf(-o));
+                l = fmaxf(o, 0.0f) - o * t + log1pf(expf(-fabsf(o)));
+                d = (p - t) / (float)n;
+            }
+            S.loss[tid] = l;
+            S.dout[tid] = d;
+        }
+        __syncthreads();
+        for (int i = tid; i < kTS * NH; i += kStepThreads) {
+            const int s = i >> 6, a = i & 63;
+            S.d2[s * kHS + a] = S.h2[s * kHS + a] > 0.0f ? S.dout[s] * S.w3[a] : 0.0f;
+        }
+        __syncthreads();
+        // d1 = W2^T d2 where layer 1 is on: samples ty + 16 i, units 4 tx + j
+        {
+            float acc[4][4] = {};
+#pragma unroll 2
+            for (int a0 = 0; a0 < NH; a0 += 4) {
+                float4 d[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) d[i] = ld4(&S.d2[(ty + 16 * i) * kHS + a0]);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const float4 w = ld4(&S.W2[(a0 + q) * kHS + 4 * tx]);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const float dq = reinterpret_cast<const float *>(&d[i])[q];
+                        acc[i][0] = fmaf(w.x, dq, acc[i][0]);
+                        acc[i][1] = fmaf(w.y, dq, acc[i][1]);
+                        acc[i][2] = fmaf(w.z, dq, acc[i][2]);
+                        acc[i][3] = fmaf(w.w, dq, acc[i][3]);
+                    }
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int at = (ty + 16 * i) * kHS + 4 * tx;
+                const float4 h = ld4(&S.h1[at]);
+                *reinterpret_cast<float4 *>(&S.d1[at]) =
+                    make_float4(h.x > 0.0f ? acc[i][0] : 0.0f, h.y > 0.0f ? acc[i][1] : 0.0f,
+                                h.z > 0.0f ? acc[i][2] : 0.0f, h.w > 0.0f ? acc[i][3] : 0.0f);
+            }
+        }
+        __syncthreads();
+        // the tile's share of the gradients: outer products over its samples
+#pragma unroll 4
+        for (int s = 0; s < kTS; ++s) {
+            const float4 d = ld4(&S.d2[s * kHS + 4 * ty]), h = ld4(&S.h1[s * kHS + 4 * tx]);
+            const float dv[4] = {d.x, d.y, d.z, d.w}, hv[4] = {h.x, h.y, h.z, h.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) g2[i][j] = fmaf(dv[i], hv[j], g2[i][j]);
+        }
+        if (tx < NF / 4) {
+#pragma unroll 4
+            for (int s = 0; s < kTS; ++s) {
+                const float4 d = ld4(&S.d1[s * kHS + 4 * ty]), h = ld4(&S.x[s * kXS + 4 * tx]);
+                const float dv[4] = {d.x, d.y, d.z, d.w}, hv[4] = {h.x, h.y, h.z, h.w};
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) g1[i][j] = fmaf(dv[i], hv[j], g1[i][j]);
+            }
+        }
+        {
+            const int q = tid >> 6, m = tid & 63;
+            if (q == 0)
+#pragma unroll 8
+                for (int s = 0; s < kTS; ++s) gv += S.d1[s * kHS + m];
+            else if (q == 1)
+#pragma unroll 8
+                for (int s = 0; s < kTS; ++s) gv += S.d2[s * kHS + m];
+            else if (q == 2)
+#pragma unroll 8
+                for (int s = 0; s < kTS; ++s) gv = fmaf(S.dout[s], S.h2[s * kHS + m], gv);
+            else if (m < 32) {  // a warp: b3 and the loss
+                float a = S.dout[m] + S.dout[m + 32], l = S.loss[m] + S.loss[m + 32];
+                for (int o = 16; o > 0; o >>= 1) {
+                    a += __shfl_xor_sync(kFull, a, o);
+                    l += __shfl_xor_sync(kFull, l, o);
+                }
+                gv += a;
+                gl += l;
+            }
+        }
+    }
+    // one row of partial sums per CTA, or the result itself when there is only one
+    float *row = gridDim.x > 1 ? out + (size_t)blockIdx.x * kPartial : out;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            row[P_W2 + (4 * ty + i) * NH + 4 * tx + j] = g2[i][j];
+            if (tx < NF / 4) row[P_W1 + (4 * ty + i) * NF + 4 * tx + j] = g1[i][j];
+        }
+    const int q = tid >> 6, m = tid & 63;
+    if (q < 3) row[(q == 0 ? P_B1 : (q == 1 ? P_B2 : P_W3)) + m] = gv;
+    if (tid == 3 * 64) {
+        row[P_B3] = gv;
+        if (gridDim.x > 1) row[NP] = gl;
+        else loss[0] = gl / (float)n;
+    }
+}
+
+// Column sums of the rows of partial sums: 32 columns per CTA, 8 threads per
+// column taking every eighth row (coalesced across the columns).
+__global__ void __launch_bounds__(256) mlp_reduce_kernel(const float *__restrict__ partial, int rows, int n,
+                                                         float *__restrict__ grad, float *__restrict__ loss)
+{
+    __shared__ float red[8][33];
+    const int c = blockIdx.x * 32 + (threadIdx.x & 31), r0 = threadIdx.x >> 5;
+    float acc = 0.0f;
+    if (c < kPartial) {
+#pragma unroll 8
+        for (int r = r0; r < rows; r += 8) acc += __ldcs(&partial[(size_t)r * kPartial + c]);
+    }
+    red[r0][threadIdx.x & 31] = acc;
+    __syncthreads();
+    if (r0 == 0 && c < kPartial) {
+        for (int k = 1; k < 8; ++k) acc += red[k][threadIdx.x];
+        if (c < NP) grad[c] = acc;
+        else loss[0] = acc / (float)n;
+    }
 }
 
 __global__ void adam_kernel(float *__restrict__ P, const float *__restrict__ g, float *__restrict__ m,
@@ -674,6 +852,20 @@ int conf_grid()
         int per = 512 / kTmemCols;
         if (regs_cta > 0) per = std::min(per, regs_sm / regs_cta);
         per = std::min(per, (int)(smem_sm / (kConfSmem + fa.sharedSizeBytes + (size_t)reserved)));
+        g = sms * std::max(per, 1);
+    }
+    return g;
+}
+
+// CTAs of mlp_step_kernel resident at once
+int step_grid()
+{
+    static int g = 0;
+    if (!g) {
+        int dev = 0, sms = 1, per = 1;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, mlp_step_kernel, kStepThreads, sizeof(StepSmem));
         g = sms * std::max(per, 1);
     }
     return g;
@@ -727,10 +919,17 @@ int itm_mlp_loss_grad(const float *params_dev, const float *feat_dev, const floa
 {
     if (n <= 0 || !params_dev || !feat_dev || !labels_dev || !scratch_dev || !grad_dev || !loss_dev) return ITM_ERR_ARG;
     cudaStream_t st = (cudaStream_t)stream;
-    cudaError_t e = cudaMemsetAsync(loss_dev, 0, sizeof(float), st);
-    if (e != cudaSuccess) return ITM_ERR_CUDA;
-    mlp_fwd_bwd_kernel<<<(n + 127) / 128, 128, 0, st>>>(params_dev, feat_dev, labels_dev, n, scratch_dev, loss_dev);
-    mlp_grad_kernel<<<(NP + 127) / 128, 128, 0, st>>>(feat_dev, scratch_dev, n, grad_dev);
+    static const cudaError_t attr =
+        cudaFuncSetAttribute(mlp_step_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(StepSmem));
+    if (attr != cudaSuccess) return check_cuda(attr);
+    // one tile per CTA up to one CTA per SM; beyond that, CTAs take several
+    // tiles in turn, and their rows of partial sums stay few
+    const int tiles = (n - 1) / kTS + 1;
+    const int grid = std::min(tiles, step_grid());
+    mlp_step_kernel<<<grid, kStepThreads, sizeof(StepSmem), st>>>(params_dev, feat_dev, labels_dev, n,
+                                                                  grid > 1 ? scratch_dev : grad_dev, loss_dev);
+    if (grid > 1)
+        mlp_reduce_kernel<<<(kPartial + 31) / 32, 256, 0, st>>>(scratch_dev, grid, n, grad_dev, loss_dev);
     return check_cuda(cudaGetLastError());
 }
 
