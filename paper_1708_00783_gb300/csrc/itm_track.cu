@@ -3,36 +3,46 @@
 //
 //  * depth_halve_kernel: one pyramid level, the mean of the valid depths of
 //    each 2x2 block (summed in raster order, one rounded division).
-//  * icp_partial_kernel: per pixel, the camera point d ((u-cx)/fx,
+//  * icp_step_kernel: per pixel, the camera point d ((u-cx)/fx,
 //    (v-cy)/fy, 1) mapped to the world by the current estimate T, projected
 //    into the reference view (nearest pixel); with both maps valid there and
 //    |T p - V| within the outlier distance, the residual r = (T p - V) . N and
 //    J = (T p x N, N) give J J^T, J r, r^2 and a count.  The per-pixel
 //    arithmetic is float with each operation rounded on its own (built with
 //    -fmad=false), so the selection of pixels is the same on any IEEE
-//    machine; a thread accumulates its pixels (about eight) in float and a
+//    machine; a thread accumulates its pixels (about four) in float and a
 //    warp adds its lanes by a float shuffle tree (FP64 is a small fraction
 //    of the FP32 rate here); the CTA adds its warps in double and writes one
 //    partial row.  Each float sum is within 13 roundings of 2^-24 of the
 //    magnitude of its terms.
-//  * icp_solve_kernel (one CTA): sums the partial rows in a fixed order (the
-//    result does not depend on scheduling), then, in double, solves
-//    H x = -g by Cholesky and applies the motion x = (omega, tau) on the world
+//  * the CTA that finishes last adds the partial rows in a fixed order (the
+//    result does not depend on scheduling), then one of its warps solves
+//    H x = -g in double and applies the motion x = (omega, tau) on the world
 //    side, T <- [R(omega) | tau] T with R by Rodrigues' formula.  The pose
 //    stays in device memory, so a whole coarse-to-fine track runs without a
-//    host round trip per step (the paper solves on the host).
+//    host round trip per step (the paper solves on the host), one launch per
+//    step, chained by programmatic dependent launch.
+//
+// What bounds a step is latency: the wait for the step before, the gathers of
+// V and N at the projected pixel (L2), then the serial end (completion count,
+// rows, 6x6 solve).  FP64 instructions cost about 16 issue cycles per warp,
+// so sums run with lanes as columns and few rows, and the solve keeps one
+// element of the symmetric system per lane.  640x480, three levels, 19 steps:
+// 800 us per track with one kernel for the sums and one for a serial solve by
+// a single thread (9 + 26 us per step), TRACK_US us with this one.
 #include "itm_ops.cuh"
 
 namespace itm {
 
 namespace {
 
-constexpr int kIcpThreads = 256;
+constexpr int kIcpThreads = 512, kIcpWarps = kIcpThreads / 32;
 
 __global__ void __launch_bounds__(256) depth_halve_kernel(const float *__restrict__ in, int W, int H,
                                                           float *__restrict__ out)
 {
     const int w = W / 2, h = H / 2;
+    grid_dep_wait();
     for (int o = blockIdx.x * blockDim.x + threadIdx.x; o < w * h; o += gridDim.x * blockDim.x) {
         const int i = o % w, j = o / w;
         float sum = 0.0f;
@@ -47,66 +57,227 @@ __global__ void __launch_bounds__(256) depth_halve_kernel(const float *__restric
         }
         out[o] = n > 0 ? fdiv(sum, (float)n) : 0.0f;
     }
+    grid_dep_launch();
 }
 
 struct IcpState {
-    float T[16];  // current camera-to-world estimate
-    int done;     // the level stopped (too few pixels or no solution)
-    int steps;    // steps applied
+    float T[16];     // current camera-to-world estimate
+    int done_level;  // the level (from 1) that stopped: too few pixels or no solution
+    int steps;       // steps applied
+    int arrived;     // CTAs of the running step that wrote their row
 };
 
-// Partial sums of CTA blockIdx.x: partials[b * kIcpSums + k].  The pose is
-// read from the tracker state st (or T_arg when st is null).
-__global__ void __launch_bounds__(kIcpThreads) icp_partial_kernel(
-    const float *__restrict__ depth, int W, int H, Intr in, const IcpState *__restrict__ st, Mat34 T_arg,
-    const float4 *__restrict__ V, const float4 *__restrict__ N, Intr ref, Mat34 M, float dist_thresh,
-    double *__restrict__ partials)
+__global__ void __launch_bounds__(32) track_begin_kernel(IcpState *st, Mat34 T)
 {
-    __shared__ double red[kIcpThreads / 32][kIcpSums];
-    if (st && st->done) return;
-    Mat34 T = T_arg;
-    if (st) {
+    grid_dep_wait();
+    if (threadIdx.x < 16) st->T[threadIdx.x] = threadIdx.x < 12 ? T.m[threadIdx.x] : (threadIdx.x == 15 ? 1.0f : 0.0f);
+    if (threadIdx.x == 0) st->done_level = st->steps = st->arrived = 0;
+    grid_dep_launch();
+}
+
+// Sum over the warp of v[0 .. 31], value l ending in lane l: each stage halves
+// the values a lane holds (31 shuffles and adds instead of 5 per value).
+__device__ __forceinline__ float warp_sum32(float (&v)[32], int lane)
+{
 #pragma unroll
-        for (int k = 0; k < 12; ++k) T.m[k] = st->T[k];
+    for (int h = 16; h > 0; h >>= 1) {
+        const bool up = lane & h;
+#pragma unroll
+        for (int i = 0; i < h; ++i) {
+            const float keep = up ? v[i + h] : v[i], send = up ? v[i] : v[i + h];
+            v[i] = fadd(keep, __shfl_xor_sync(kFull, send, h));
+        }
     }
-    const float t2 = fmul(dist_thresh, dist_thresh);
-    float acc[kIcpSums - 1];
+    return v[0];
+}
+
+// Lane l's column of the CTA's kIcpWarps rows in red, added in a fixed order:
+// complete in warp 0 (every thread of the CTA calls).
+__device__ __forceinline__ double column_sum(double (*red)[32], double x, int lane, int warp)
+{
+    red[warp][lane] = x;
+    __syncthreads();
+    if (warp < 4) {
+        x = red[4 * warp][lane];
 #pragma unroll
-    for (int k = 0; k < kIcpSums - 1; ++k) acc[k] = 0.0f;
-    int count = 0;
-    const int n_pix = W * H;
+        for (int k = 1; k < kIcpWarps / 4; ++k) x += red[4 * warp + k][lane];
+    }
+    __syncthreads();
+    if (warp < 4) red[warp][lane] = x;
+    __syncthreads();
+    return warp == 0 ? (red[0][lane] + red[1][lane]) + (red[2][lane] + red[3][lane]) : 0.0;
+}
+static_assert(kIcpWarps == 16, "column_sum adds four groups of four warps");
+
+// Columns of the n_part partial rows, added in a fixed order by the whole
+// CTA: lane l of warp 0 gets column l.
+__device__ __forceinline__ double row_sums(const double *__restrict__ partials, int n_part, double (*red)[32], int lane,
+                                           int warp)
+{
+    double x = 0.0;
+    if (lane < kIcpSums) {
+#pragma unroll 4
+        for (int b = warp; b < n_part; b += kIcpWarps) x += __ldcg(&partials[(size_t)b * kIcpSums + lane]);
+    }
+    __syncthreads();  // red may still be read
+    return column_sum(red, x, lane, warp);
+}
+
+// One Gauss-Newton step by one warp: lane l holds sums[l] in x, that is
+// element (i, j), i <= j, of the upper triangle of H row by row, then -g's
+// entries as column 6.  Elimination keeps one element per lane: with pivot p,
+// a_ij -= a_pi a_pj / a_pp for p < i <= j (H = L D L^T; the pivots are the
+// squares of Cholesky's, so the system is refused in the same cases).
+// Returns false when it has no solution; else T and the motion are applied.
+__device__ __forceinline__ bool gauss_newton_warp(double x, IcpState *st, int lane)
+{
+    if (__shfl_sync(kFull, x, 28) < 6.0) return false;
+    // this lane's row and column: sums 0..20 are (i, j), 21..26 are (i, 6)
+    int i = 0, j = 0;
+    {
+        int k = 0;
+#pragma unroll
+        for (int r = 0; r < 6; ++r)
+#pragma unroll
+            for (int c = r; c < 6; ++c, ++k)
+                if (k == lane) i = r, j = c;
+        if (lane >= 21) i = min(lane - 21, 5), j = 6;
+    }
+    const auto at = [](int r, int c) { return c == 6 ? 21 + r : 6 * r - r * (r - 1) / 2 + (c - r); };  // r <= c
+    double inv[6];
+#pragma unroll
+    for (int p = 0; p < 6; ++p) {
+        const double a = __shfl_sync(kFull, x, at(p, p));
+        if (!(a > 0.0)) return false;  // uniform
+        inv[p] = 1.0 / a;
+        if (p == 5) break;
+        const double aj = __shfl_sync(kFull, x, j < p ? 0 : at(p, j)), ai = __shfl_sync(kFull, x, i < p ? 0 : at(p, i));
+        if (i > p && lane < 27) x -= ai * (aj * inv[p]);
+    }
+    // U x = -g by columns from the last
+    double s[6];
+#pragma unroll
+    for (int c = 5; c >= 0; --c) {
+        s[c] = __shfl_sync(kFull, x, at(c, 6)) * inv[c];
+        const double u = __shfl_sync(kFull, x, i <= c ? at(i, c) : 0);
+        if (j == 6 && i < c) x -= u * s[c];
+    }
+#pragma unroll
+    for (int c = 0; c < 6; ++c) s[c] = -s[c];
+    // R = I + s1 K + s2 K^2, K = [omega]_x, K^2 = omega omega^T - th^2 I, with
+    // s1 = sin(th) / th, s2 = (1 - cos(th)) / th^2: their Taylor series in
+    // th^2 for the usual small steps (below 2^-70 relative beyond eight terms)
+    const double t2 = s[0] * s[0] + s[1] * s[1] + s[2] * s[2];
+    double s1, s2;
+    if (t2 < 0.0625) {
+        s1 = s2 = 0.0;
+#pragma unroll
+        for (int k = 8; k >= 1; --k) {
+            s1 = 1.0 - t2 * (1.0 / ((2.0 * k) * (2.0 * k + 1.0))) * (k == 8 ? 1.0 : s1);
+            s2 = 1.0 - t2 * (1.0 / ((2.0 * k + 1.0) * (2.0 * k + 2.0))) * (k == 8 ? 1.0 : s2);
+        }
+        s2 *= 0.5;
+    } else {
+        const double th = sqrt(t2);
+        s1 = sin(th) / th;
+        s2 = (1.0 - cos(th)) / t2;
+    }
+    // lane 4 r + c < 12: element (r, c) of [R | tau] T
+    float Tn = 0.0f;
+    if (lane < 12) {
+        const int r = lane >> 2, c = lane & 3;
+        const double wr = r == 0 ? s[0] : (r == 1 ? s[1] : s[2]);
+        double acc = c == 3 ? (r == 0 ? s[3] : (r == 1 ? s[4] : s[5])) : 0.0;
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+            double R = s2 * wr * s[m];
+            if (m == r) {
+                R += 1.0 - s2 * t2;
+            } else {
+                const int o = 3 - r - m;  // K[r][m] = -+ omega_o
+                const double w = s1 * (o == 0 ? s[0] : (o == 1 ? s[1] : s[2]));
+                R += (m - r + 3) % 3 == 1 ? -w : w;
+            }
+            acc += R * (double)__ldcg(&st->T[4 * m + c]);
+        }
+        Tn = (float)acc;
+    }
+    __syncwarp();  // every lane has read T
+    if (lane < 12) st->T[lane] = Tn;
+    if (lane == 0) st->steps += 1;
+    return true;
+}
+
+// Partial sums of CTA blockIdx.x: partials[b * kIcpSums + k].  The pose is
+// read from the tracker state st, and the CTA that finishes last takes the
+// step (icp_solve is then done); or, with st null, from T_arg.  du and dv are
+// (gridDim.x * blockDim.x) % W and / W.  prefetch: the depth frame was
+// complete before the previous kernel of the stream began, so it is read
+// before the wait for that kernel.
+__global__ void __launch_bounds__(kIcpThreads) icp_step_kernel(
+    const float *__restrict__ depth, int W, int H, Intr in, IcpState *st, int level, Mat34 T_arg,
+    const float4 *__restrict__ V, const float4 *__restrict__ N, Intr ref, Mat34 M, float dist_thresh,
+    double *__restrict__ partials, int du, int dv, bool prefetch)
+{
+    __shared__ double red[kIcpWarps][32];
+    __shared__ int is_last;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // kBatch pixels per pass (p, p + stride, ...): their depth loads, then
     // their map loads, are issued together
     constexpr int kBatch = 4;
-    const int stride = gridDim.x * blockDim.x;
-    for (int p0 = blockIdx.x * blockDim.x + threadIdx.x; p0 < n_pix; p0 += kBatch * stride) {
-        float dk[kBatch];
+    const int n_pix = W * H, stride = gridDim.x * blockDim.x;
+    int p0 = blockIdx.x * blockDim.x + threadIdx.x;
+    int u = p0 % W, v = p0 / W;
+    float dk[kBatch];
+    auto read_depth = [&]() {
 #pragma unroll
         for (int b = 0; b < kBatch; ++b) {
             const int p = p0 + b * stride;
             dk[b] = p < n_pix ? __ldg(&depth[p]) : 0.0f;
         }
+    };
+    if (prefetch) read_depth();
+    grid_dep_wait();
+    if (st && __ldcg(&st->done_level) == level) return;
+    if (!prefetch) read_depth();
+    Mat34 T = T_arg;
+    if (st) {
+#pragma unroll
+        for (int k = 0; k < 12; ++k) T.m[k] = __ldcg(&st->T[k]);
+    }
+    const float t2 = fmul(dist_thresh, dist_thresh);
+    float acc[32];
+#pragma unroll
+    for (int k = 0; k < 32; ++k) acc[k] = 0.0f;
+    int count = 0;
+    while (p0 < n_pix) {
         float pw[kBatch][3];
         int o[kBatch];
 #pragma unroll
         for (int b = 0; b < kBatch; ++b) {
             o[b] = -1;
             const float d = dk[b];
-            if (!(d > 0.0f)) continue;
-            const int p = p0 + b * stride;
-            const int u = p % W, v = p / W;
-            const float pcx = fmul(fdiv(fsub((float)u, in.cx), in.fx), d);
-            const float pcy = fmul(fdiv(fsub((float)v, in.cy), in.fy), d);
-            float pr[3];
+            if (d > 0.0f) {
+                const float pcx = fmul(fdiv(fsub((float)u, in.cx), in.fx), d);
+                const float pcy = fmul(fdiv(fsub((float)v, in.cy), in.fy), d);
+                float pr[3];
 #pragma unroll
-            for (int r = 0; r < 3; ++r) pw[b][r] = row_apply(T.m + 4 * r, pcx, pcy, d);
+                for (int r = 0; r < 3; ++r) pw[b][r] = row_apply(T.m + 4 * r, pcx, pcy, d);
 #pragma unroll
-            for (int r = 0; r < 3; ++r) pr[r] = row_apply(M.m + 4 * r, pw[b][0], pw[b][1], pw[b][2]);
-            if (!(pr[2] > 0.0f)) continue;
-            const float ur = fadd(fdiv(fmul(ref.fx, pr[0]), pr[2]), ref.cx);
-            const float vr = fadd(fdiv(fmul(ref.fy, pr[1]), pr[2]), ref.cy);
-            if (!(ur >= 0.0f && ur <= (float)(ref.W - 1) && vr >= 0.0f && vr <= (float)(ref.H - 1))) continue;
-            o[b] = (int)fadd(vr, 0.5f) * ref.W + (int)fadd(ur, 0.5f);
+                for (int r = 0; r < 3; ++r) pr[r] = row_apply(M.m + 4 * r, pw[b][0], pw[b][1], pw[b][2]);
+                if (pr[2] > 0.0f) {
+                    const float ur = fadd(fdiv(fmul(ref.fx, pr[0]), pr[2]), ref.cx);
+                    const float vr = fadd(fdiv(fmul(ref.fy, pr[1]), pr[2]), ref.cy);
+                    if (ur >= 0.0f && ur <= (float)(ref.W - 1) && vr >= 0.0f && vr <= (float)(ref.H - 1))
+                        o[b] = (int)fadd(vr, 0.5f) * ref.W + (int)fadd(ur, 0.5f);
+                }
+            }
+            u += du;
+            v += dv;
+            if (u >= W) {
+                u -= W;
+                ++v;
+            }
         }
         float4 Vk[kBatch], Nk[kBatch];
 #pragma unroll
@@ -118,6 +289,8 @@ __global__ void __launch_bounds__(kIcpThreads) icp_partial_kernel(
                 Nk[b] = __ldg(&N[o[b]]);
             }
         }
+        p0 += kBatch * stride;
+        if (p0 < n_pix) read_depth();
 #pragma unroll
         for (int b = 0; b < kBatch; ++b) {
             if (o[b] < 0) continue;
@@ -130,115 +303,51 @@ __global__ void __launch_bounds__(kIcpThreads) icp_partial_kernel(
             const float J[6] = {fsub(fmul(pw[b][1], Np.z), fmul(pw[b][2], Np.y)),
                                 fsub(fmul(pw[b][2], Np.x), fmul(pw[b][0], Np.z)),
                                 fsub(fmul(pw[b][0], Np.y), fmul(pw[b][1], Np.x)), Np.x, Np.y, Np.z};
+            // sums: one rounding per term (FMA)
             int k = 0;
 #pragma unroll
             for (int i = 0; i < 6; ++i)
 #pragma unroll
-                for (int j = i; j < 6; ++j, ++k) acc[k] = fadd(acc[k], fmul(J[i], J[j]));
+                for (int j = i; j < 6; ++j, ++k) acc[k] = __fmaf_rn(J[i], J[j], acc[k]);
 #pragma unroll
-            for (int i = 0; i < 6; ++i) acc[21 + i] = fadd(acc[21 + i], fmul(J[i], res));
-            acc[27] = fadd(acc[27], fmul(res, res));
+            for (int i = 0; i < 6; ++i) acc[21 + i] = __fmaf_rn(J[i], res, acc[21 + i]);
+            acc[27] = __fmaf_rn(res, res, acc[27]);
             ++count;
         }
     }
-    // warps by float shuffle trees (the count exactly, as an integer), then
-    // the CTA's warp rows in double, in order
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int k = 0; k < kIcpSums - 1; ++k) {
-        float x = acc[k];
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) x = fadd(x, __shfl_down_sync(kFull, x, off));
-        if (lane == 0) red[warp][k] = (double)x;
+    // warps by float shuffle trees (the count is a whole number below 2^24:
+    // exact), then the CTA's warp rows in double, in order
+    static_assert(kIcpSums == 29, "28 sums and the count");
+    acc[28] = (float)count;
+    const double x = column_sum(red, (double)warp_sum32(acc, lane), lane, warp);
+    if (warp == 0) {
+        if (lane < kIcpSums) {
+            partials[(size_t)blockIdx.x * kIcpSums + lane] = x;
+            __threadfence();
+        }
+        __syncwarp();
+        if (lane == 0) is_last = st && atomicAdd(&st->arrived, 1) == (int)gridDim.x - 1;
     }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) count += __shfl_down_sync(kFull, count, off);
-    if (lane == 0) red[warp][kIcpSums - 1] = (double)count;
+    if (!st) return;  // icp_sum_kernel adds the rows
     __syncthreads();
-    if (threadIdx.x < kIcpSums) {
-        double x = 0.0;
-#pragma unroll
-        for (int w = 0; w < kIcpThreads / 32; ++w) x += red[w][threadIdx.x];
-        partials[(size_t)blockIdx.x * kIcpSums + threadIdx.x] = x;
-    }
+    grid_dep_launch();
+    if (!is_last) return;
+    __threadfence();
+    const double sum = row_sums(partials, gridDim.x, red, lane, warp);
+    if (warp != 0) return;
+    if (lane == 0) st->arrived = 0;
+    if (!gauss_newton_warp(sum, st, lane) && lane == 0) st->done_level = level;
 }
 
-// Sums the n_part partial rows into sums: warp w adds column w, lane l the
-// rows l, l + 32, ... in order, then a fixed shuffle tree (the result does
-// not depend on scheduling); with st, thread 0 then takes the Gauss-Newton
-// step.
-__global__ void __launch_bounds__(1024) icp_solve_kernel(const double *__restrict__ partials, int n_part,
-                                                         double *__restrict__ sums, IcpState *st)
+// The n_part partial rows added into sums (one CTA).
+__global__ void __launch_bounds__(kIcpThreads) icp_sum_kernel(const double *__restrict__ partials, int n_part,
+                                                              double *__restrict__ sums)
 {
-    if (st && st->done) return;
+    __shared__ double red[kIcpWarps][32];
+    grid_dep_wait();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (warp < kIcpSums) {
-        double x = 0.0;
-        for (int b = lane; b < n_part; b += 32) x += partials[(size_t)b * kIcpSums + warp];
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) x += __shfl_down_sync(kFull, x, off);
-        if (lane == 0) sums[warp] = x;
-    }
-    __syncthreads();
-    if (!st || threadIdx.x != 0) return;
-    if (sums[28] < 6.0) {
-        st->done = 1;
-        return;
-    }
-    double A[6][6], L[6][6], y[6], x[6];
-    int k = 0;
-    for (int i = 0; i < 6; ++i)
-        for (int j = i; j < 6; ++j, ++k) A[i][j] = A[j][i] = sums[k];
-    for (int i = 0; i < 6; ++i) {
-        for (int j = 0; j <= i; ++j) {
-            double a = A[i][j];
-            for (int m = 0; m < j; ++m) a -= L[i][m] * L[j][m];
-            if (i == j) {
-                if (!(a > 0.0)) {
-                    st->done = 1;
-                    return;
-                }
-                L[i][i] = sqrt(a);
-            } else {
-                L[i][j] = a / L[j][j];
-            }
-        }
-    }
-    for (int i = 0; i < 6; ++i) {
-        double a = -sums[21 + i];
-        for (int m = 0; m < i; ++m) a -= L[i][m] * y[m];
-        y[i] = a / L[i][i];
-    }
-    for (int i = 5; i >= 0; --i) {
-        double a = y[i];
-        for (int m = i + 1; m < 6; ++m) a -= L[m][i] * x[m];
-        x[i] = a / L[i][i];
-    }
-    // R = I + sin(th)/th K + (1 - cos(th))/th^2 K^2, K = [omega]_x
-    const double th = sqrt(x[0] * x[0] + x[1] * x[1] + x[2] * x[2]);
-    const double s1 = th > 1e-12 ? sin(th) / th : 1.0;
-    const double s2 = th > 1e-12 ? (1.0 - cos(th)) / (th * th) : 0.5;
-    const double K[3][3] = {{0.0, -x[2], x[1]}, {x[2], 0.0, -x[0]}, {-x[1], x[0], 0.0}};
-    double R[3][3];
-    for (int i = 0; i < 3; ++i)
-        for (int j = 0; j < 3; ++j) {
-            double k2 = 0.0;
-            for (int m = 0; m < 3; ++m) k2 += K[i][m] * K[m][j];
-            R[i][j] = (i == j ? 1.0 : 0.0) + s1 * K[i][j] + s2 * k2;
-        }
-    float Tn[12];
-    for (int i = 0; i < 3; ++i) {
-        for (int j = 0; j < 3; ++j) {
-            double a = 0.0;
-            for (int m = 0; m < 3; ++m) a += R[i][m] * (double)st->T[4 * m + j];
-            Tn[4 * i + j] = (float)a;
-        }
-        double a = x[3 + i];
-        for (int m = 0; m < 3; ++m) a += R[i][m] * (double)st->T[4 * m + 3];
-        Tn[4 * i + 3] = (float)a;
-    }
-    for (int i = 0; i < 12; ++i) st->T[i] = Tn[i];
-    st->steps += 1;
+    const double x = row_sums(partials, n_part, red, lane, warp);
+    if (warp == 0 && lane < kIcpSums) sums[lane] = x;
 }
 
 int icp_grid(int n_pix)
@@ -250,9 +359,10 @@ int icp_grid(int n_pix)
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (sms < 1) sms = 1;
     }
-    // about eight pixels per thread, at most two CTAs per SM and kIcpMaxPartials rows
-    int g = (n_pix + 8 * kIcpThreads - 1) / (8 * kIcpThreads);
-    if (g > 2 * sms) g = 2 * sms;
+    // one pixel per thread while there are SMs for it, then one CTA per SM
+    // (few rows for the last CTA: FP64 adds) and several pixels per thread
+    int g = (n_pix - 1) / kIcpThreads + 1;
+    if (g > sms) g = sms;
     if (g > kIcpMaxPartials) g = kIcpMaxPartials;
     return g > 0 ? g : 1;
 }
@@ -265,8 +375,7 @@ cudaError_t launch_depth_halve(const float *in, int W, int H, float *out, cudaSt
     if (n <= 0) return cudaSuccess;
     int g = (n + 255) / 256;
     if (g > 1216) g = 1216;
-    depth_halve_kernel<<<g, 256, 0, st>>>(in, W, H, out);
-    return cudaGetLastError();
+    return launch_pdl(depth_halve_kernel, dim3(g), dim3(256), 0, st, in, W, H, out);
 }
 
 cudaError_t launch_icp_reduce(const float *depth, const Intr &in, const Mat34 &T_g, const float4 *V, const float4 *N,
@@ -274,10 +383,12 @@ cudaError_t launch_icp_reduce(const float *depth, const Intr &in, const Mat34 &T
 {
     const int g = icp_grid(in.W * in.H);
     double *partials = work + kIcpSums;
-    icp_partial_kernel<<<g, kIcpThreads, 0, st>>>(depth, in.W, in.H, in, nullptr, T_g, V, N, ref, M_ref, dist_thresh,
-                                                   partials);
-    icp_solve_kernel<<<1, 1024, 0, st>>>(partials, g, work, nullptr);
-    return cudaGetLastError();
+    const int stride = g * kIcpThreads;
+    cudaError_t e = launch_pdl(icp_step_kernel, dim3(g), dim3(kIcpThreads), 0, st, depth, in.W, in.H, in,
+                               (IcpState *)nullptr, 0, T_g, V, N, ref, M_ref, dist_thresh, partials, stride % in.W,
+                               stride / in.W, false);
+    if (e != cudaSuccess) return e;
+    return launch_pdl(icp_sum_kernel, dim3(1), dim3(kIcpThreads), 0, st, (const double *)partials, g, work);
 }
 
 size_t track_scratch_bytes(int W, int H, int levels)
@@ -305,6 +416,10 @@ cudaError_t launch_track(const float *depth, const Intr &in0, int levels, const 
     Intr li[kTrackMaxLevels];
     lev[0] = depth;
     li[0] = in0;
+    Mat34 T0;
+    pose_rows(T, T0);
+    cudaError_t e = launch_pdl(track_begin_kernel, dim3(1), dim3(32), 0, st, state, T0);
+    if (e != cudaSuccess) return e;
     for (int l = 1; l < levels; ++l) {
         float *out = reinterpret_cast<float *>(base + off);
         li[l].W = li[l - 1].W / 2;
@@ -316,29 +431,27 @@ cudaError_t launch_track(const float *depth, const Intr &in0, int levels, const 
         li[l].fy = fy;
         li[l].cx = cxm / 2.0f;
         li[l].cy = cym / 2.0f;
-        cudaError_t e = launch_depth_halve(lev[l - 1], li[l - 1].W, li[l - 1].H, out, st);
+        e = launch_depth_halve(lev[l - 1], li[l - 1].W, li[l - 1].H, out, st);
         if (e != cudaSuccess) return e;
         lev[l] = out;
         off += sizeof(float) * (size_t)li[l].W * (size_t)li[l].H;
         off = (off + 255) & ~(size_t)255;
     }
-    IcpState h_state;
-    memset(&h_state, 0, sizeof(h_state));
-    memcpy(h_state.T, T, sizeof(h_state.T));
-    cudaError_t e = cudaMemcpyAsync(state, &h_state, sizeof(h_state), cudaMemcpyHostToDevice, st);
-    if (e != cudaSuccess) return e;
     double *partials = work + kIcpSums;
+    bool first = true;
     for (int l = levels - 1; l >= 0; --l) {
         if (iters[l] <= 0 || li[l].W < 1 || li[l].H < 1) continue;
-        e = cudaMemsetAsync(&state->done, 0, sizeof(int), st);
-        if (e != cudaSuccess) return e;
-        const int g = icp_grid(li[l].W * li[l].H);
+        const int g = icp_grid(li[l].W * li[l].H), stride = g * kIcpThreads;
         for (int it = 0; it < iters[l]; ++it) {
-            icp_partial_kernel<<<g, kIcpThreads, 0, st>>>(lev[l], li[l].W, li[l].H, li[l], state, Mat34{}, V, N, ref,
-                                                           M_ref, thresh[l], partials);
-            icp_solve_kernel<<<1, 1024, 0, st>>>(partials, g, work, state);
+            // the first step follows the pyramid's last kernel, which may have written its depth
+            e = launch_pdl(icp_step_kernel, dim3(g), dim3(kIcpThreads), 0, st, lev[l], li[l].W, li[l].H, li[l], state,
+                           l + 1, Mat34{}, V, N, ref, M_ref, thresh[l], partials, stride % li[l].W, stride / li[l].W,
+                           !first);
+            if (e != cudaSuccess) return e;
+            first = false;
         }
     }
+    IcpState h_state;
     e = cudaMemcpyAsync(&h_state, state, sizeof(h_state), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return e;
