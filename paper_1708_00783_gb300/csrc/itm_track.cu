@@ -29,7 +29,8 @@
 // so sums run with lanes as columns and few rows, and the solve keeps one
 // element of the symmetric system per lane.  640x480, three levels, 19 steps:
 // 800 us per track with one kernel for the sums and one for a serial solve by
-// a single thread (9 + 26 us per step), TRACK_US us with this one.
+// a single thread (9 + 26 us per step), 330 us with this one (362 with IEEE divisions in
+// the solve and two divisions per pixel for its ray).
 #include "itm_ops.cuh"
 
 namespace itm {
@@ -37,6 +38,7 @@ namespace itm {
 namespace {
 
 constexpr int kIcpThreads = 512, kIcpWarps = kIcpThreads / 32;
+constexpr int kBatch = 4;  // pixels of a thread per pass
 
 __global__ void __launch_bounds__(256) depth_halve_kernel(const float *__restrict__ in, int W, int H,
                                                           float *__restrict__ out)
@@ -116,11 +118,33 @@ __device__ __forceinline__ double row_sums(const double *__restrict__ partials, 
 {
     double x = 0.0;
     if (lane < kIcpSums) {
-#pragma unroll 4
-        for (int b = warp; b < n_part; b += kIcpWarps) x += __ldcg(&partials[(size_t)b * kIcpSums + lane]);
+        // ten rows at a time (152 CTAs: one pass), their loads issued together
+        for (int b0 = warp; b0 < n_part; b0 += 10 * kIcpWarps) {
+            double r[10];
+#pragma unroll
+            for (int k = 0; k < 10; ++k) {
+                const int b = b0 + k * kIcpWarps;
+                r[k] = b < n_part ? __ldcg(&partials[(size_t)b * kIcpSums + lane]) : 0.0;
+            }
+#pragma unroll
+            for (int k = 0; k < 10; ++k)
+                if (b0 + k * kIcpWarps < n_part) x += r[k];  // uniform over the warp
+        }
     }
     __syncthreads();  // red may still be read
     return column_sum(red, x, lane, warp);
+}
+
+// 1 / a to within an ulp of double: Newton's iteration y + y (1 - a y) from
+// the float reciprocal, whose error 2^-23 it squares twice (four FP64
+// operations; the IEEE division costs several times as many).
+__device__ __forceinline__ double rcp_double(double a)
+{
+    const float f = (float)a;
+    if (!(f > 0x1p-100f && f < 0x1p100f)) return 1.0 / a;
+    double y = (double)__frcp_rn(f);
+    y = __fma_rn(y, __fma_rn(-a, y, 1.0), y);
+    return __fma_rn(y, __fma_rn(-a, y, 1.0), y);
 }
 
 // One Gauss-Newton step by one warp: lane l holds sums[l] in x, that is
@@ -149,10 +173,10 @@ __device__ __forceinline__ bool gauss_newton_warp(double x, IcpState *st, int la
     for (int p = 0; p < 6; ++p) {
         const double a = __shfl_sync(kFull, x, at(p, p));
         if (!(a > 0.0)) return false;  // uniform
-        inv[p] = 1.0 / a;
+        inv[p] = rcp_double(a);
         if (p == 5) break;
         const double aj = __shfl_sync(kFull, x, j < p ? 0 : at(p, j)), ai = __shfl_sync(kFull, x, i < p ? 0 : at(p, i));
-        if (i > p && lane < 27) x -= ai * (aj * inv[p]);
+        if (i > p && lane < 27) x = __fma_rn(-ai, aj * inv[p], x);
     }
     // U x = -g by columns from the last
     double s[6];
@@ -160,23 +184,32 @@ __device__ __forceinline__ bool gauss_newton_warp(double x, IcpState *st, int la
     for (int c = 5; c >= 0; --c) {
         s[c] = __shfl_sync(kFull, x, at(c, 6)) * inv[c];
         const double u = __shfl_sync(kFull, x, i <= c ? at(i, c) : 0);
-        if (j == 6 && i < c) x -= u * s[c];
+        if (j == 6 && i < c) x = __fma_rn(-u, s[c], x);
     }
 #pragma unroll
     for (int c = 0; c < 6; ++c) s[c] = -s[c];
     // R = I + s1 K + s2 K^2, K = [omega]_x, K^2 = omega omega^T - th^2 I, with
     // s1 = sin(th) / th, s2 = (1 - cos(th)) / th^2: their Taylor series in
-    // th^2 for the usual small steps (below 2^-70 relative beyond eight terms)
-    const double t2 = s[0] * s[0] + s[1] * s[1] + s[2] * s[2];
+    // th^2 for the usual small steps, to below 2^-60 relative (th < 1/64: the
+    // term t2^4 / 9! is the last above it; th < 1/4: t2^7 / 15!)
+    const double t2 = __fma_rn(s[0], s[0], __fma_rn(s[1], s[1], s[2] * s[2]));
     double s1, s2;
-    if (t2 < 0.0625) {
-        s1 = s2 = 0.0;
-#pragma unroll
-        for (int k = 8; k >= 1; --k) {
-            s1 = 1.0 - t2 * (1.0 / ((2.0 * k) * (2.0 * k + 1.0))) * (k == 8 ? 1.0 : s1);
-            s2 = 1.0 - t2 * (1.0 / ((2.0 * k + 1.0) * (2.0 * k + 2.0))) * (k == 8 ? 1.0 : s2);
+    if (t2 < 0x1p-4) {
+        constexpr double c1[8] = {1.0, -1.0 / 6, 1.0 / 120, -1.0 / 5040, 1.0 / 362880, -1.0 / 39916800,
+                                  1.0 / 6227020800.0, -1.0 / 1307674368000.0};
+        constexpr double c2[8] = {1.0 / 2, -1.0 / 24, 1.0 / 720, -1.0 / 40320, 1.0 / 3628800, -1.0 / 479001600,
+                                  1.0 / 87178291200.0, -1.0 / 20922789888000.0};
+        s1 = c1[4];
+        s2 = c2[4];
+        if (t2 >= 0x1p-12) {
+            s1 = __fma_rn(t2, __fma_rn(t2, __fma_rn(t2, c1[7], c1[6]), c1[5]), c1[4]);
+            s2 = __fma_rn(t2, __fma_rn(t2, __fma_rn(t2, c2[7], c2[6]), c2[5]), c2[4]);
         }
-        s2 *= 0.5;
+#pragma unroll
+        for (int k = 3; k >= 0; --k) {
+            s1 = __fma_rn(t2, s1, c1[k]);
+            s2 = __fma_rn(t2, s2, c2[k]);
+        }
     } else {
         const double th = sqrt(t2);
         s1 = sin(th) / th;
@@ -186,19 +219,16 @@ __device__ __forceinline__ bool gauss_newton_warp(double x, IcpState *st, int la
     float Tn = 0.0f;
     if (lane < 12) {
         const int r = lane >> 2, c = lane & 3;
+        const float Tc[3] = {__ldcg(&st->T[c]), __ldcg(&st->T[4 + c]), __ldcg(&st->T[8 + c])};
         const double wr = r == 0 ? s[0] : (r == 1 ? s[1] : s[2]);
         double acc = c == 3 ? (r == 0 ? s[3] : (r == 1 ? s[4] : s[5])) : 0.0;
 #pragma unroll
         for (int m = 0; m < 3; ++m) {
-            double R = s2 * wr * s[m];
-            if (m == r) {
-                R += 1.0 - s2 * t2;
-            } else {
-                const int o = 3 - r - m;  // K[r][m] = -+ omega_o
-                const double w = s1 * (o == 0 ? s[0] : (o == 1 ? s[1] : s[2]));
-                R += (m - r + 3) % 3 == 1 ? -w : w;
-            }
-            acc += R * (double)__ldcg(&st->T[4 * m + c]);
+            const int o = 3 - r - m;  // off the diagonal, K[r][m] = -+ omega_o
+            const double w = o == 0 ? s[0] : (o == 1 ? s[1] : s[2]);
+            const double k = m == r ? -s2 * t2 : ((m - r + 3) % 3 == 1 ? -s1 : s1) * w;
+            const double R = __fma_rn(s2 * wr, s[m], m == r ? 1.0 + k : k);
+            acc = __fma_rn(R, (double)Tc[m], acc);
         }
         Tn = (float)acc;
     }
@@ -210,30 +240,29 @@ __device__ __forceinline__ bool gauss_newton_warp(double x, IcpState *st, int la
 
 // Partial sums of CTA blockIdx.x: partials[b * kIcpSums + k].  The pose is
 // read from the tracker state st, and the CTA that finishes last takes the
-// step (icp_solve is then done); or, with st null, from T_arg.  du and dv are
-// (gridDim.x * blockDim.x) % W and / W.  prefetch: the depth frame was
+// step; or, with st null, from T_arg.  A thread takes pixels of one column, up
+// to kBatch of them rows rows apart (rows = ceil(H / batch): one division for
+// the column's ray, and the pixels of a warp still lie side by side): position
+// p of W x rows stands for pixels (p % W, p / W + b rows).  prefetch: the depth frame was
 // complete before the previous kernel of the stream began, so it is read
 // before the wait for that kernel.
 __global__ void __launch_bounds__(kIcpThreads) icp_step_kernel(
     const float *__restrict__ depth, int W, int H, Intr in, IcpState *st, int level, Mat34 T_arg,
     const float4 *__restrict__ V, const float4 *__restrict__ N, Intr ref, Mat34 M, float dist_thresh,
-    double *__restrict__ partials, int du, int dv, bool prefetch)
+    double *__restrict__ partials, int rows, bool prefetch)
 {
     __shared__ double red[kIcpWarps][32];
     __shared__ int is_last;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    // kBatch pixels per pass (p, p + stride, ...): their depth loads, then
-    // their map loads, are issued together
-    constexpr int kBatch = 4;
-    const int n_pix = W * H, stride = gridDim.x * blockDim.x;
+    // a pass's depth loads, then its map loads, are issued together
+    const int n_pos = W * rows, stride = gridDim.x * blockDim.x;
     int p0 = blockIdx.x * blockDim.x + threadIdx.x;
-    int u = p0 % W, v = p0 / W;
     float dk[kBatch];
     auto read_depth = [&]() {
 #pragma unroll
         for (int b = 0; b < kBatch; ++b) {
-            const int p = p0 + b * stride;
-            dk[b] = p < n_pix ? __ldg(&depth[p]) : 0.0f;
+            const int p = p0 + b * n_pos;  // row-major: b rows rows further down
+            dk[b] = p0 < n_pos && p < W * H ? __ldg(&depth[p]) : 0.0f;
         }
     };
     if (prefetch) read_depth();
@@ -250,7 +279,9 @@ __global__ void __launch_bounds__(kIcpThreads) icp_step_kernel(
 #pragma unroll
     for (int k = 0; k < 32; ++k) acc[k] = 0.0f;
     int count = 0;
-    while (p0 < n_pix) {
+    while (p0 < n_pos) {
+        const int u = p0 % W, v = p0 / W;
+        const float rx = fdiv(fsub((float)u, in.cx), in.fx);
         float pw[kBatch][3];
         int o[kBatch];
 #pragma unroll
@@ -258,8 +289,8 @@ __global__ void __launch_bounds__(kIcpThreads) icp_step_kernel(
             o[b] = -1;
             const float d = dk[b];
             if (d > 0.0f) {
-                const float pcx = fmul(fdiv(fsub((float)u, in.cx), in.fx), d);
-                const float pcy = fmul(fdiv(fsub((float)v, in.cy), in.fy), d);
+                const float pcx = fmul(rx, d);
+                const float pcy = fmul(fdiv(fsub((float)(v + b * rows), in.cy), in.fy), d);
                 float pr[3];
 #pragma unroll
                 for (int r = 0; r < 3; ++r) pw[b][r] = row_apply(T.m + 4 * r, pcx, pcy, d);
@@ -272,12 +303,6 @@ __global__ void __launch_bounds__(kIcpThreads) icp_step_kernel(
                         o[b] = (int)fadd(vr, 0.5f) * ref.W + (int)fadd(ur, 0.5f);
                 }
             }
-            u += du;
-            v += dv;
-            if (u >= W) {
-                u -= W;
-                ++v;
-            }
         }
         float4 Vk[kBatch], Nk[kBatch];
 #pragma unroll
@@ -289,8 +314,8 @@ __global__ void __launch_bounds__(kIcpThreads) icp_step_kernel(
                 Nk[b] = __ldg(&N[o[b]]);
             }
         }
-        p0 += kBatch * stride;
-        if (p0 < n_pix) read_depth();
+        p0 += stride;
+        read_depth();
 #pragma unroll
         for (int b = 0; b < kBatch; ++b) {
             if (o[b] < 0) continue;
@@ -350,7 +375,10 @@ __global__ void __launch_bounds__(kIcpThreads) icp_sum_kernel(const double *__re
     if (warp == 0 && lane < kIcpSums) sums[lane] = x;
 }
 
-int icp_grid(int n_pix)
+// Rows of a step's positions and its CTAs: one pixel per thread while there
+// are SMs for it (latency), then up to kBatch per thread and one CTA per SM
+// (few partial rows for the last CTA to add in FP64).
+int icp_shape(int W, int H, int &rows)
 {
     static int sms = 0;
     if (!sms) {
@@ -359,12 +387,13 @@ int icp_grid(int n_pix)
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (sms < 1) sms = 1;
     }
-    // one pixel per thread while there are SMs for it, then one CTA per SM
-    // (few rows for the last CTA: FP64 adds) and several pixels per thread
-    int g = (n_pix - 1) / kIcpThreads + 1;
-    if (g > sms) g = sms;
-    if (g > kIcpMaxPartials) g = kIcpMaxPartials;
-    return g > 0 ? g : 1;
+    const int most = sms < kIcpMaxPartials ? sms : kIcpMaxPartials;
+    int batch = 1;
+    do
+        rows = (H + batch - 1) / batch;
+    while ((long long)W * rows > (long long)most * kIcpThreads && batch++ < kBatch);
+    const int g = (W * rows - 1) / kIcpThreads + 1;
+    return g < most ? g : most;
 }
 
 }  // namespace
@@ -381,12 +410,11 @@ cudaError_t launch_depth_halve(const float *in, int W, int H, float *out, cudaSt
 cudaError_t launch_icp_reduce(const float *depth, const Intr &in, const Mat34 &T_g, const float4 *V, const float4 *N,
                               const Intr &ref, const Mat34 &M_ref, float dist_thresh, double *work, cudaStream_t st)
 {
-    const int g = icp_grid(in.W * in.H);
+    int rows = 0;
+    const int g = icp_shape(in.W, in.H, rows);
     double *partials = work + kIcpSums;
-    const int stride = g * kIcpThreads;
     cudaError_t e = launch_pdl(icp_step_kernel, dim3(g), dim3(kIcpThreads), 0, st, depth, in.W, in.H, in,
-                               (IcpState *)nullptr, 0, T_g, V, N, ref, M_ref, dist_thresh, partials, stride % in.W,
-                               stride / in.W, false);
+                               (IcpState *)nullptr, 0, T_g, V, N, ref, M_ref, dist_thresh, partials, rows, false);
     if (e != cudaSuccess) return e;
     return launch_pdl(icp_sum_kernel, dim3(1), dim3(kIcpThreads), 0, st, (const double *)partials, g, work);
 }
@@ -441,12 +469,12 @@ cudaError_t launch_track(const float *depth, const Intr &in0, int levels, const 
     bool first = true;
     for (int l = levels - 1; l >= 0; --l) {
         if (iters[l] <= 0 || li[l].W < 1 || li[l].H < 1) continue;
-        const int g = icp_grid(li[l].W * li[l].H), stride = g * kIcpThreads;
+        int rows = 0;
+        const int g = icp_shape(li[l].W, li[l].H, rows);
         for (int it = 0; it < iters[l]; ++it) {
             // the first step follows the pyramid's last kernel, which may have written its depth
             e = launch_pdl(icp_step_kernel, dim3(g), dim3(kIcpThreads), 0, st, lev[l], li[l].W, li[l].H, li[l], state,
-                           l + 1, Mat34{}, V, N, ref, M_ref, thresh[l], partials, stride % li[l].W, stride / li[l].W,
-                           !first);
+                           l + 1, Mat34{}, V, N, ref, M_ref, thresh[l], partials, rows, !first);
             if (e != cudaSuccess) return e;
             first = false;
         }
