@@ -22,7 +22,9 @@
 //     image with z > 0 and lie within the frame's depth range + mu is
 //     appended to the visible list (Sec. 4.2, third part); eight lanes per
 //     block, one per corner.  When the raycast will use the allocation pose,
-//     the same pass also rasterises each block's search range.
+//     the same pass also rasterises each block's search range.  It also enters
+//     the blocks this allocation handed out (a few dozen in a usual frame) in
+//     the brick table.
 //
 // Counts produced on the device are read by the next kernel from device
 // memory (persistent grid-stride loops), so no host synchronisation and no
@@ -78,10 +80,11 @@ __global__ void __launch_bounds__(256) build_visible_kernel(SceneDev s, Mat34 M,
     grid_dep_wait();
     const int n = min(__ldcg(&s.ctr->block_head), s.nv);
     const float zfar = visible_zfar(s);
+    const int brick_from = __ldcg(&s.ctr->brick_from);
     const int groups = gridDim.x * (blockDim.x >> 3);
     for (int g0 = blockIdx.x * (blockDim.x >> 3); g0 < n; g0 += groups) {
         const int i = g0 + (threadIdx.x >> 3);
-        visible_8<false>(s, M, in, zfar, i < n, i, 0.0f, 1, 1);
+        visible_8<false>(s, M, in, zfar, brick_from, i < n, i, 0.0f, 1, 1);
     }
     grid_dep_launch();
 }
@@ -94,10 +97,11 @@ __global__ void __launch_bounds__(256) build_visible_range_kernel(SceneDev s, Ma
     grid_dep_wait();
     const int n = min(__ldcg(&s.ctr->block_head), s.nv);
     const float zfar = visible_zfar(s);
+    const int brick_from = __ldcg(&s.ctr->brick_from);
     const int groups = gridDim.x * (blockDim.x >> 3);
     for (int g0 = blockIdx.x * (blockDim.x >> 3); g0 < n; g0 += groups) {
         const int i = g0 + (threadIdx.x >> 3);
-        visible_8<true>(s, M, in, zfar, i < n, i, zc, tiles_x, tiles_y);
+        visible_8<true>(s, M, in, zfar, brick_from, i < n, i, zc, tiles_x, tiles_y);
     }
     grid_dep_launch();
 }
@@ -128,9 +132,7 @@ cudaError_t launch_allocate(const SceneDev &s, const float *depth, const Intr &i
                             const Mat34 &M_d, bool with_range, cudaStream_t st, const uint16_t *raw)
 {
     static_assert(kFrameCountersOffset % 4 == 0 && kFrameCountersBytes % 4 == 0, "word-aligned frame counters");
-    cudaError_t e = launch_pdl(zero_words_kernel, dim3(1), dim3(32), 0, st,
-                               reinterpret_cast<int32_t *>(reinterpret_cast<char *>(s.ctr) + kFrameCountersOffset),
-                               (int)(kFrameCountersBytes / 4));
+    cudaError_t e = launch_pdl(alloc_begin_kernel, dim3(1), dim3(32), 0, st, s.ctr);
     if (e != cudaSuccess) return e;
     const float inv_b = (float)(1.0 / (8.0 * (double)s.voxel_size));
     dim3 grid((in.W + 31) / 32, (in.H + 7) / 8);

@@ -99,6 +99,7 @@ __global__ void __launch_bounds__(256) batch_begin_kernel(const ItemDev *__restr
     const ItemDev &it = items[blockIdx.x];
     if (threadIdx.x < kFrameCountersBytes / 4)
         reinterpret_cast<int *>(reinterpret_cast<char *>(it.s.ctr) + kFrameCountersOffset)[threadIdx.x] = 0;
+    if (threadIdx.x == 31) it.s.ctr->brick_from = it.s.ctr->block_head;
     const int tiles = it.rtiles_x * it.rtiles_y;
     for (int i = threadIdx.x; i < tiles; i += blockDim.x) {
         it.s.range_min[i] = 0xffffffffu;

@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(256) colour_at_kernel(SceneDev s, const float4
             if (coord_ok(q[0]) && coord_ok(q[1]) && coord_ok(q[2])) {
                 const int gx = (int)floorf(fadd(q[0], 0.5f)), gy = (int)floorf(fadd(q[1], 0.5f));
                 const int gz = (int)floorf(fadd(q[2], 0.5f));
-                const int ptr = lookup_ro(s, gx >> 3, gy >> 3, gz >> 3);
+                const int ptr = brick_find(s, gx >> 3, gy >> 3, gz >> 3);
                 if (ptr >= 0) c = __ldg(&rgbw[(size_t)ptr * kBlockVoxels + (gx & 7) + 8 * (gy & 7) + 64 * (gz & 7)]);
             }
         }

@@ -89,17 +89,8 @@ __device__ __forceinline__ void trilinear_fw(const SceneDev &s, const float (&q)
     const float g0x = floorf(q[0]), g0y = floorf(q[1]), g0z = floorf(q[2]);
     const float fx = fsub(q[0], g0x), fy = fsub(q[1], g0y), fz = fsub(q[2], g0z);
     const int x = (int)g0x, y = (int)g0y, z = (int)g0z;
-    const int bx = x >> 3, by = y >> 3, bz = z >> 3;
-    const bool cx = (x & 7) == 7, cy = (y & 7) == 7, cz = (z & 7) == 7;
     int P[8];
-    P[0] = lookup_ro(s, bx, by, bz);
-    P[1] = cx ? lookup_ro(s, bx + 1, by, bz) : P[0];
-    P[2] = cy ? lookup_ro(s, bx, by + 1, bz) : P[0];
-    P[3] = cy ? (cx ? lookup_ro(s, bx + 1, by + 1, bz) : P[2]) : P[1];
-    P[4] = cz ? lookup_ro(s, bx, by, bz + 1) : P[0];
-    P[5] = cz ? (cx ? lookup_ro(s, bx + 1, by, bz + 1) : P[4]) : P[1];
-    P[6] = cz ? (cy ? lookup_ro(s, bx, by + 1, bz + 1) : P[4]) : P[2];
-    P[7] = cz ? (cy ? (cx ? lookup_ro(s, bx + 1, by + 1, bz + 1) : P[6]) : P[5]) : P[3];
+    brick_fetch8(s, x >> 3, y >> 3, z >> 3, (x & 7) == 7, (y & 7) == 7, (z & 7) == 7, P);
     const int lx[2] = {x & 7, (x + 1) & 7};
     const int ly[2] = {8 * (y & 7), 8 * ((y + 1) & 7)};
     const int lz[2] = {64 * (z & 7), 64 * ((z + 1) & 7)};
@@ -156,7 +147,7 @@ __device__ __forceinline__ bool combined_alloc(const CombinedArgs &A, const floa
         const int bx = ((int)floorf(fadd(q[0], 0.5f))) >> 3;
         const int by = ((int)floorf(fadd(q[1], 0.5f))) >> 3;
         const int bz = ((int)floorf(fadd(q[2], 0.5f))) >> 3;
-        if (in_i16(bx) && in_i16(by) && in_i16(bz) && lookup_ro(A.sub[i], bx, by, bz) >= 0) return true;
+        if (in_i16(bx) && in_i16(by) && in_i16(bz) && brick_find(A.sub[i], bx, by, bz) >= 0) return true;
     }
     return false;
 }

@@ -71,7 +71,40 @@ __global__ void reset_blocks_kernel(SceneDev s)
     }
 }
 
+// Empties the places that were taken (a warp each; the others are empty: a
+// scene clears its whole table once, when it is made).
+__global__ void __launch_bounds__(256) brick_reset_kernel(SceneDev s)
+{
+    const int lane = threadIdx.x & 31;
+    const uint32_t warps = gridDim.x * (blockDim.x >> 5);
+    for (uint32_t p = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); p <= s.brick_mask; p += warps) {
+        if (s.brick_owner[p] == 0ull) continue;  // uniform over the warp
+        __syncwarp();
+        int4 *cell = reinterpret_cast<int4 *>(s.brick_cell + (size_t)p * kBrickCells);
+        for (int i = lane; i < kBrickCells / 4; i += 32) cell[i] = make_int4(-1, -1, -1, -1);
+        if (lane == 0) {
+            s.brick_owner[p] = 0ull;
+            s.brick_count[p] = 0;
+        }
+    }
+}
+
+__global__ void __launch_bounds__(256) brick_fill_kernel(SceneDev s, int n)
+{
+    for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < 8ll * n; j += (long long)gridDim.x * blockDim.x) {
+        const short4 b = s.block_pos[j >> 3];
+        if (b.w) brick_put(s, b.x, b.y, b.z, (int)(j >> 3), (int)(j & 7));
+    }
+}
+
 }  // namespace
+
+cudaError_t launch_brick_fill(const SceneDev &s, int n, cudaStream_t st)
+{
+    if (n <= 0) return cudaSuccess;
+    brick_fill_kernel<<<stream_grid(), 256, 0, st>>>(s, n);
+    return cudaGetLastError();
+}
 
 cudaError_t launch_depth_u16(const uint16_t *raw, float *out, int64_t n, cudaStream_t st)
 {
@@ -86,6 +119,7 @@ cudaError_t launch_reset(const SceneDev &s, cudaStream_t st)
 {
     reset_entries_kernel<<<stream_grid(), 256, 0, st>>>(s);
     if (s.nv > 0) reset_blocks_kernel<<<stream_grid(), 256, 0, st>>>(s);
+    brick_reset_kernel<<<stream_grid(), 256, 0, st>>>(s);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     return cudaMemsetAsync(s.ctr, 0, sizeof(Counters), st);

@@ -12,6 +12,8 @@
 //   block_free  int32[nv]           free block list, handed out front to back
 //   excess_free int32[ne]           free excess slots, handed out front to back
 //   ctr         Counters            device counters and the sticky status word
+//   brick_*     per brick place     block indices by block coordinates (brick_fetch8), for the
+//                                   kernels that only look blocks up
 //   swap_state  uint8[nb + ne]      Sec. 5 swapping (itm_swap_enable): kSw* per entry
 //   touch       int32[nv]           last allocation whose segments met the block (-1: freed
 //                                   by the running swap-out)
@@ -72,6 +74,7 @@ struct Counters {
     unsigned long long visited;  // cumulative voxels visited by integration
     unsigned long long frames;   // cumulative integrated frames
     unsigned long long mesh_tris;  // per-mesh: triangles found
+    int32_t brick_from;  // per-frame: blocks handed out before it (they are in the brick table)
 };
 
 // Offset and size of the per-frame counters cleared at the start of allocation.
@@ -92,6 +95,10 @@ struct SceneDev {
     int32_t *block_free;
     int32_t *excess_free;
     Counters *ctr;
+    unsigned long long *brick_owner;  // the brick of each place (brick_key), 0: none yet
+    int32_t *brick_count;             // cells of the place that hold a block
+    int32_t *brick_cell;              // kBrickCells block indices per place, -1: none
+    uint32_t brick_mask;              // places - 1
     uint32_t *range_min;  // per 8x4 tile: nearest / farthest depth (float bits) of covering blocks
     uint32_t *range_max;
     // raycast tile queues, two sides (one written by a raycast, the other
@@ -198,6 +205,182 @@ __device__ __forceinline__ int lookup_cg(const SceneDev &s, int bx, int by, int 
     return -1;
 }
 
+// ----------------------------------------------------------- brick table
+// The blocks in device memory by their coordinates, for the kernels that look
+// blocks up without changing them (the raycasts, the mesh, the colour of
+// points): beside the hash table, which stays what decides.  A brick is 8 x 8
+// x 8 blocks, brick (X, Y, Z) = (bx, by, bz) >> 3; its place in the table is a
+// hash of its coordinates.  A place has room for one brick, the first that
+// came (brick_owner), and holds 9 x 9 x 9 block indices: the brick's blocks
+// and the blocks one further along each axis, so that the up to eight blocks
+// that a 2x2x2 voxel stencil reaches are cells of one brick at fixed offsets.
+// Blocks of a brick whose place is taken are not entered; the place is marked
+// (kBrickShared) and lookups in that brick go to the hash table.
+//
+// Why: through the hash table each of those eight blocks was a key, a hash
+// and a scattered 16-byte load of its own, one after the other wherever any
+// lane of the warp crossed a block face; here they are 4-byte loads of
+// neighbouring words that are issued together with the owner's, so that a
+// sample has two dependent loads, cells and voxels.  (Neighbour indices kept
+// with each block, found through the hash, made three and measured slower:
+// 153 us against 151 us before and 129 us now for a 640x480 frame of
+// the room; cells with a tag of their own instead of the place's owner took a
+// fifth more instructions.)
+//
+// Blocks enter in the visible pass after the allocation that handed them out
+// (and after an import), and leave in the swap-out; the kernels that change
+// the table and those that read it never run at the same time.
+constexpr int kBrickSide = 9;      // blocks along a brick's edge with the one further
+constexpr int kBrickCells = 736;   // 9^3 cells, rounded up to whole 32-byte sectors
+constexpr int kBrickMin = 4096;    // smallest number of places (12 MB)
+constexpr unsigned long long kBrickValid = 1ull << 48, kBrickShared = 1ull << 63;
+
+// places for nv blocks: one for every 16 blocks (a surface fills a brick with
+// about a hundred, and the bricks before it by their ninth cells), 184 bytes
+// per block beside its 2560 bytes of voxels.  Bricks that find their place
+// taken cost the walks the table is there to save: with one place for 32
+// blocks, 512 at least, a camera turning round in a room of 350 bricks took
+// 196 us per frame instead of 168.
+inline int brick_places(int nv)
+{
+    int n = kBrickMin;
+    while (n < nv / 16) n *= 2;
+    return n;
+}
+
+// the owner word of brick (X, Y, Z) = block coordinates >> 3
+__host__ __device__ __forceinline__ unsigned long long brick_key(int X, int Y, int Z)
+{
+    return (unsigned long long)((uint32_t)(X & 0xffff) | ((uint32_t)Y << 16)) |
+           ((unsigned long long)((uint32_t)(Z & 0xffff) | 0x10000u) << 32);
+}
+// its place: neighbouring bricks lie apart from each other, distant ones at random
+__host__ __device__ __forceinline__ uint32_t brick_place(int X, int Y, int Z, uint32_t mask)
+{
+    return ((uint32_t)X + (uint32_t)Y * 0x9e3779b1u + (uint32_t)Z * 0x85ebca77u) & mask;
+}
+__host__ __device__ __forceinline__ int brick_local(int lx, int ly, int lz)
+{
+    return lx + kBrickSide * ly + kBrickSide * kBrickSide * lz;
+}
+
+// The hash table's answers for the stencil of a brick whose place is shared
+// (bit k of want: the block at dx + 2 dy + 4 dz = k is asked for).
+static __device__ __noinline__ int lookup_chain(const SceneDev &s, int bx, int by, int bz)
+{
+    return lookup_ro(s, bx, by, bz);
+}
+
+// The block index at (bx, by, bz), or -1.
+__device__ __forceinline__ int brick_find(const SceneDev &s, int bx, int by, int bz)
+{
+    const int X = bx >> 3, Y = by >> 3, Z = bz >> 3;
+    const uint32_t place = brick_place(X, Y, Z, s.brick_mask);
+    const unsigned long long own = __ldg(&s.brick_owner[place]), key = brick_key(X, Y, Z);
+    const int p = __ldg(&s.brick_cell[(size_t)place * kBrickCells + brick_local(bx & 7, by & 7, bz & 7)]);
+    if ((own & ~kBrickShared) == key) return ITM_IN_BOUNDS(s, p < s.nv) ? p : -1;
+    return own & kBrickShared ? lookup_chain(s, bx, by, bz) : -1;
+}
+
+// The blocks of the 2x2x2 neighbourhood of block (bx, by, bz) towards +x, +y,
+// +z: P[dx + 2 dy + 4 dz], where an axis without its cross flag stays at the
+// block itself.
+__device__ __forceinline__ void brick_fetch8(const SceneDev &s, int bx, int by, int bz, bool cx, bool cy, bool cz,
+                                             int (&P)[8])
+{
+    const int X = bx >> 3, Y = by >> 3, Z = bz >> 3;
+    const uint32_t place = brick_place(X, Y, Z, s.brick_mask);
+    const int32_t *cell = s.brick_cell + (size_t)place * kBrickCells + brick_local(bx & 7, by & 7, bz & 7);
+    const unsigned long long own = __ldg(&s.brick_owner[place]), key = brick_key(X, Y, Z);
+    constexpr int dx = 1, dy = kBrickSide, dz = kBrickSide * kBrickSide;
+    int R[8];
+    R[0] = __ldg(cell);
+#pragma unroll
+    for (int k = 1; k < 8; ++k) {
+        R[k] = -1;
+        if ((!(k & 1) || cx) && (!(k & 2) || cy) && (!(k & 4) || cz))
+            R[k] = __ldg(cell + ((k & 1) ? dx : 0) + ((k & 2) ? dy : 0) + ((k & 4) ? dz : 0));
+    }
+    if ((own & ~kBrickShared) != key) {
+        // no block of this brick is in the table: none exists, or they are only in the hash table
+        const bool chain = (own & kBrickShared) != 0ull;
+        const int skip = (cx ? 0 : 1) | (cy ? 0 : 2) | (cz ? 0 : 4);
+#pragma unroll 1
+        for (int k = 0; k < 8; ++k) {
+            const int p = chain && !(k & skip) ? lookup_chain(s, bx + (k & 1), by + ((k >> 1) & 1), bz + (k >> 2)) : -1;
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                if (j == k) R[j] = p;
+        }
+    }
+#ifdef ITM_CHECK_BOUNDS
+    for (int k = 0; k < 8; ++k)
+        if (!ITM_IN_BOUNDS(s, R[k] < s.nv)) R[k] = -1;
+#endif
+    P[0] = R[0];
+    P[1] = cx ? R[1] : R[0];
+    P[2] = cy ? R[2] : R[0];
+    P[3] = cy ? (cx ? R[3] : R[2]) : P[1];
+    P[4] = cz ? R[4] : R[0];
+    P[5] = cz ? (cx ? R[5] : R[4]) : P[1];
+    P[6] = cz ? (cy ? R[6] : R[4]) : P[2];
+    P[7] = cz ? (cy ? (cx ? R[7] : R[6]) : P[5]) : P[3];
+}
+
+// Block (bx, by, bz) is a cell of its own brick and, on each axis where it is
+// the brick's first, the ninth cell of the brick before: c = 0..7 takes the
+// brick that is one before on the axes of c's bits.  False when there is no
+// such brick (also outside the int16 block coordinates).
+__host__ __device__ __forceinline__ bool brick_share(int bx, int by, int bz, int c, int &X, int &Y, int &Z, int &local)
+{
+    int b[3] = {bx, by, bz}, B[3], l[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        B[i] = b[i] >> 3;
+        l[i] = b[i] & 7;
+        if (c & (1 << i)) {
+            if (l[i] != 0 || B[i] == -4096) return false;
+            B[i] -= 1;
+            l[i] = 8;
+        }
+    }
+    X = B[0];
+    Y = B[1];
+    Z = B[2];
+    local = brick_local(l[0], l[1], l[2]);
+    return true;
+}
+
+// Block ptr enters at (bx, by, bz): the share of lane or thread c (0..7).
+__device__ __forceinline__ void brick_put(const SceneDev &s, int bx, int by, int bz, int ptr, int c)
+{
+    int X, Y, Z, local;
+    if (!brick_share(bx, by, bz, c, X, Y, Z, local)) return;
+    const uint32_t place = brick_place(X, Y, Z, s.brick_mask);
+    const unsigned long long key = brick_key(X, Y, Z);
+    const unsigned long long old = atomicCAS(&s.brick_owner[place], 0ull, key);
+    if (old == 0ull || (old & ~kBrickShared) == key) {
+        s.brick_cell[(size_t)place * kBrickCells + local] = ptr;
+        atomicAdd(&s.brick_count[place], 1);
+    } else {
+        atomicOr(&s.brick_owner[place], kBrickShared);
+    }
+}
+
+// The block at (bx, by, bz) leaves: the share of thread c (0..7).  A place
+// whose last block leaves is free again; a shared one never is (blocks of
+// other bricks may only be in the hash table).
+__device__ __forceinline__ void brick_take(const SceneDev &s, int bx, int by, int bz, int c)
+{
+    int X, Y, Z, local;
+    if (!brick_share(bx, by, bz, c, X, Y, Z, local)) return;
+    const uint32_t place = brick_place(X, Y, Z, s.brick_mask);
+    const unsigned long long own = __ldcg(&s.brick_owner[place]);
+    if ((own & ~kBrickShared) != brick_key(X, Y, Z)) return;
+    s.brick_cell[(size_t)place * kBrickCells + local] = -1;
+    if (atomicSub(&s.brick_count[place], 1) == 1 && !(own & kBrickShared)) s.brick_owner[place] = 0ull;
+}
+
 // ------------------------------------------------------ slab partition
 // Block column x belongs to part floor(x / w) mod n; a part keeps its own
 // columns and kShardGhost columns on either side (whose voxels every sample
@@ -254,6 +437,18 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
 }
 
 namespace {
+// The start of an allocation: its counters cleared, the blocks handed out so
+// far noted (they are in the brick table).  A kernel of the chain and not a
+// memset, which would break it.
+__global__ void __launch_bounds__(32) alloc_begin_kernel(Counters *ctr)
+{
+    grid_dep_wait();
+    if (threadIdx.x < kFrameCountersBytes / 4)
+        reinterpret_cast<int32_t *>(reinterpret_cast<char *>(ctr) + kFrameCountersOffset)[threadIdx.x] = 0;
+    if (threadIdx.x == 31) ctr->brick_from = ctr->block_head;
+    grid_dep_launch();
+}
+
 // Zeroes n 32-bit words at p after the previous kernel (a launch_pdl stand-in
 // for cudaMemsetAsync, which would break the chain of dependent launches).
 __global__ void __launch_bounds__(32) zero_words_kernel(int32_t *p, int n)
@@ -383,4 +578,6 @@ cudaError_t launch_depth_u16(const uint16_t *raw, float *out, int64_t n, cudaStr
 cudaError_t launch_raycast_merge(const float4 *vtx, const float4 *nrm, int parts, long long npix, const Mat34 &M_d,
                                  float4 *vo, float4 *no, cudaStream_t st);
 cudaError_t launch_reset(const SceneDev &s, cudaStream_t st);
+// enters blocks 0 .. n-1 (block_pos) in the brick table
+cudaError_t launch_brick_fill(const SceneDev &s, int n, cudaStream_t st);
 }  // namespace itm

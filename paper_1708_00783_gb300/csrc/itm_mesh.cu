@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(kMeshThreads) mesh_kernel(SceneDev s, const Mc
         if (threadIdx.x < 8) {
             const int t = threadIdx.x;
             const int bx = b.x + (t & 1), by = b.y + ((t >> 1) & 1), bz = b.z + (t >> 2);
-            P[t] = t == 0 ? ptr : (in_i16(bx) && in_i16(by) && in_i16(bz) ? lookup_ro(s, bx, by, bz) : -1);
+            P[t] = t == 0 ? ptr : (in_i16(bx) && in_i16(by) && in_i16(bz) ? brick_find(s, bx, by, bz) : -1);
         }
         __syncthreads();
         for (int v = threadIdx.x; v < kHalo * kHalo * kHalo; v += blockDim.x) {

@@ -92,7 +92,7 @@ static void free_dev(SceneDev &d)
 {
     void *ptrs[] = {d.entries, d.req, d.req_list, d.overflow, d.visible, d.block_pos, d.sdf,
                     d.w8, d.w32, d.block_free, d.excess_free, d.ctr, d.range_min, d.range_max,
-                    d.tile_q_hdr, d.tile_q_list};
+                    d.tile_q_hdr, d.tile_q_list, d.brick_owner, d.brick_count, d.brick_cell};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     memset(&d, 0, sizeof(d));
@@ -165,6 +165,11 @@ int itm_scene_create(const itm_scene_params *params, itm_scene **out)
     ITM_ALLOC(d.block_free, sizeof(int32_t) * (size_t)(d.nv > 0 ? d.nv : 1));
     ITM_ALLOC(d.excess_free, sizeof(int32_t) * (size_t)(d.ne > 0 ? d.ne : 1));
     ITM_ALLOC(d.ctr, sizeof(Counters));
+    const size_t places = (size_t)brick_places(d.nv);
+    d.brick_mask = (uint32_t)(places - 1);
+    ITM_ALLOC(d.brick_owner, sizeof(unsigned long long) * places);
+    ITM_ALLOC(d.brick_count, sizeof(int32_t) * places);
+    ITM_ALLOC(d.brick_cell, sizeof(int32_t) * kBrickCells * places);
     ITM_ALLOC(d.range_min, sizeof(uint32_t) * (size_t)kRangeMaxTiles);
     ITM_ALLOC(d.range_max, sizeof(uint32_t) * (size_t)kRangeMaxTiles);
     ITM_ALLOC(d.tile_q_hdr, sizeof(int32_t) * 2 * kTileHdrInts);
@@ -175,6 +180,9 @@ int itm_scene_create(const itm_scene_params *params, itm_scene **out)
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&sc->ev_fork, cudaEventDisableTiming);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&sc->ev_join, cudaEventDisableTiming);
     }
+    if (e == cudaSuccess) e = cudaMemsetAsync(d.brick_owner, 0, sizeof(unsigned long long) * places, 0);
+    if (e == cudaSuccess) e = cudaMemsetAsync(d.brick_count, 0, sizeof(int32_t) * places, 0);
+    if (e == cudaSuccess) e = cudaMemsetAsync(d.brick_cell, 0xff, sizeof(int32_t) * kBrickCells * places, 0);
     if (e == cudaSuccess) e = launch_reset(d, 0);
     if (e == cudaSuccess) e = cudaStreamSynchronize(0);
     if (e != cudaSuccess) {
@@ -773,8 +781,11 @@ int itm_scene_import(itm_scene *sc, const int16_t *coords_host, const float *sdf
         memset(&c, 0, sizeof(c));
         c.block_head = n;
         c.excess_head = used_excess;
+        c.brick_from = n;
         e = cudaMemcpy(d.ctr, &c, sizeof(c), cudaMemcpyHostToDevice);
     }
+    if (e == cudaSuccess) e = launch_brick_fill(d, n, 0);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(0);
     sc->last_stream = 0;
     return check_cuda(e);
 }

@@ -301,6 +301,10 @@ __global__ void __launch_bounds__(kMoveThreads) swap_out_kernel(SceneDev s, Swap
         const int idx = s_idx, ptr = s_ptr;
         __syncthreads();
         if (ptr < 0) continue;  // uniform over the CTA
+        if (t < 8) {
+            const Entry &E = s.entries[idx];
+            brick_take(s, E.x, E.y, E.z, t);
+        }
         float4 *F = reinterpret_cast<float4 *>(s.sdf + (size_t)ptr * kBlockVoxels);
         float4 *HF = reinterpret_cast<float4 *>(w.host_sdf + (size_t)idx * kBlockVoxels);
         HF[t] = __ldcg(&F[t]);
