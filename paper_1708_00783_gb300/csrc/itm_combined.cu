@@ -81,16 +81,13 @@ __global__ void __launch_bounds__(256) combined_range_kernel(const CombinedArgs 
     }
 }
 
-// Trilinear interpolation of the sdf and of the weight of submap s at its
-// voxel coordinates q (|q| < 262000); unallocated voxels: sdf 1, weight 0.
+// Trilinear interpolation of the sdf and of the weight of submap s at voxel
+// coordinates with floor (x, y, z) and fractions (fx, fy, fz), P the blocks of
+// the eight voxels; unallocated voxels: sdf 1, weight 0.
 template <int MODE>
-__device__ __forceinline__ void trilinear_fw(const SceneDev &s, const float (&q)[3], float &F, float &Wt)
+__device__ __forceinline__ void trilinear_fw(const SceneDev &s, const int (&P)[8], int x, int y, int z, float fx,
+                                             float fy, float fz, float &F, float &Wt)
 {
-    const float g0x = floorf(q[0]), g0y = floorf(q[1]), g0z = floorf(q[2]);
-    const float fx = fsub(q[0], g0x), fy = fsub(q[1], g0y), fz = fsub(q[2], g0z);
-    const int x = (int)g0x, y = (int)g0y, z = (int)g0z;
-    int P[8];
-    brick_fetch8(s, x >> 3, y >> 3, z >> 3, (x & 7) == 7, (y & 7) == 7, (z & 7) == 7, P);
     const int lx[2] = {x & 7, (x + 1) & 7};
     const int ly[2] = {8 * (y & 7), 8 * ((y + 1) & 7)};
     const int lz[2] = {64 * (z & 7), 64 * ((z + 1) & 7)};
@@ -136,36 +133,91 @@ __device__ __forceinline__ bool submap_coords(const CombinedArgs &A, int i, cons
     return ok;
 }
 
-// Is the block of the voxel nearest to X (ray depth t) allocated in some submap?
-__device__ __forceinline__ bool combined_alloc(const CombinedArgs &A, const float (&X)[3], float inv_s, float t,
-                                               const float *lo, const float *hi)
-{
-    for (int i = 0; i < A.n; ++i) {
-        if (!in_range(A, lo, hi, i, t)) continue;
-        float q[3];
-        if (!submap_coords(A, i, X, inv_s, q)) continue;
-        const int bx = ((int)floorf(fadd(q[0], 0.5f))) >> 3;
-        const int by = ((int)floorf(fadd(q[1], 0.5f))) >> 3;
-        const int bz = ((int)floorf(fadd(q[2], 0.5f))) >> 3;
-        if (in_i16(bx) && in_i16(by) && in_i16(bz) && brick_find(A.sub[i], bx, by, bz) >= 0) return true;
-    }
-    return false;
-}
-
-// The combined value at X; den receives the weight sum.  With ray depth t
-// (on_ray) submaps whose range misses t are skipped (their term is 0).
-template <int MODE>
-__device__ __forceinline__ float combined_value(const CombinedArgs &A, const float (&X)[3], float inv_s, float &den,
-                                                bool on_ray = false, float t = 0.0f, const float *lo = nullptr,
-                                                const float *hi = nullptr)
+// The combined map at the ray's sample X (ray depth t): whether the block of
+// the voxel nearest to it is allocated in some submap and, unless only that is
+// asked (COARSE), the value and the weight sum.  One set of blocks per submap
+// answers both (the nearest voxel lies in the stencil, as in the raycast of
+// one scene); a submap whose range misses t, or with no block in the stencil,
+// contributes exact zeros and is skipped.
+template <int MODE, bool COARSE_ONLY>
+__device__ __forceinline__ bool combined_sample(const CombinedArgs &A, const float (&X)[3], float inv_s, float t,
+                                                const float *lo, const float *hi, float &F, float &den)
 {
     float num = 0.0f, dsum = 0.0f;
+    bool alloc = false;
     for (int i = 0; i < A.n; ++i) {
-        if (on_ray && !in_range(A, lo, hi, i, t)) continue;
+        if (!in_range(A, lo, hi, i, t)) continue;
+        float q[3], f[3];
+        if (!submap_coords(A, i, X, inv_s, q)) continue;
+        int g[3], P[8];
+        bool c[3], up[3];
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+            const float gf = floorf(q[r]);
+            g[r] = (int)gf;
+            f[r] = fsub(q[r], gf);
+            c[r] = (g[r] & 7) == 7;
+            up[r] = c[r] && fadd(q[r], 0.5f) >= fadd(gf, 1.0f);
+        }
+        if (COARSE_ONLY) {
+            if (brick_find(A.sub[i], (g[0] >> 3) + up[0], (g[1] >> 3) + up[1], (g[2] >> 3) + up[2]) >= 0) return true;
+            continue;
+        }
+        brick_fetch8(A.sub[i], g[0] >> 3, g[1] >> 3, g[2] >> 3, c[0], c[1], c[2], P);
+        alloc = alloc || sel_block(P, up[0], up[1], up[2]) >= 0;
+        if (max(max(max(P[0], P[1]), max(P[2], P[3])), max(max(P[4], P[5]), max(P[6], P[7]))) < 0) continue;
+        float Fi, Wi;
+        trilinear_fw<MODE>(A.sub[i], P, g[0], g[1], g[2], f[0], f[1], f[2], Fi, Wi);
+        num = fadd(num, fmul(Wi, Fi));
+        dsum = fadd(dsum, Wi);
+    }
+    den = dsum;
+    F = dsum > 0.0f ? fdiv(num, dsum) : 1.0f;
+    return alloc;
+}
+
+// The submaps (bits) with a block near X: those without one within three
+// voxels of X's cell contribute exact zeros to a sample within one voxel of X.
+__device__ __forceinline__ unsigned submaps_near(const CombinedArgs &A, const float (&X)[3], float inv_s)
+{
+    unsigned near = 0;
+    for (int i = 0; i < A.n; ++i) {
+        float q[3];
+        int b[3], B[8];
+        bool c[3];
+        // a sample out of range there may be in range a voxel away: kept
+        if (!submap_coords(A, i, X, inv_s, q)) {
+            near |= 1u << i;
+            continue;
+        }
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+            const int g = (int)floorf(q[r]);
+            b[r] = (g - 2) >> 3;
+            c[r] = ((g + 3) >> 3) != b[r];
+        }
+        brick_fetch8(A.sub[i], b[0], b[1], b[2], c[0], c[1], c[2], B);
+        if (max(max(max(B[0], B[1]), max(B[2], B[3])), max(max(B[4], B[5]), max(B[6], B[7]))) >= 0) near |= 1u << i;
+    }
+    return near;
+}
+
+// The combined value at X over the submaps of the mask; den: the weight sum.
+template <int MODE>
+__device__ __forceinline__ float combined_value(const CombinedArgs &A, const float (&X)[3], float inv_s, unsigned mask,
+                                                float &den)
+{
+    float num = 0.0f, dsum = 0.0f;
+    for (; mask; mask &= mask - 1) {
+        const int i = __ffs(mask) - 1;
         float q[3];
         if (!submap_coords(A, i, X, inv_s, q)) continue;
+        const float g0 = floorf(q[0]), g1 = floorf(q[1]), g2 = floorf(q[2]);
+        const int x = (int)g0, y = (int)g1, z = (int)g2;
+        int P[8];
+        brick_fetch8(A.sub[i], x >> 3, y >> 3, z >> 3, (x & 7) == 7, (y & 7) == 7, (z & 7) == 7, P);
         float F, Wt;
-        trilinear_fw<MODE>(A.sub[i], q, F, Wt);
+        trilinear_fw<MODE>(A.sub[i], P, x, y, z, fsub(q[0], g0), fsub(q[1], g1), fsub(q[2], g2), F, Wt);
         num = fadd(num, fmul(Wt, F));
         dsum = fadd(dsum, Wt);
     }
@@ -232,9 +284,9 @@ __global__ void __launch_bounds__(256) raycast_combined_kernel(const CombinedArg
         if (A.use_range && state != SURFACE && t > T1) break;  // only unallocated space ahead: a miss
 #pragma unroll
         for (int i = 0; i < 3; ++i) X[i] = fadd(org[i], fmul(t, dir[i]));
-        const bool alloc = combined_alloc(A, X, inv_s, t, lo, hi);
+        float F, den;
         if (state == COARSE) {
-            if (!alloc) {
+            if (!combined_sample<MODE, true>(A, X, inv_s, t, lo, hi, F, den)) {
                 t = fadd(t, tB);
             } else {
                 t = fsub(t, tB);
@@ -242,13 +294,11 @@ __global__ void __launch_bounds__(256) raycast_combined_kernel(const CombinedArg
             }
             continue;
         }
-        if (!alloc) {
+        if (!combined_sample<MODE, false>(A, X, inv_s, t, lo, hi, F, den)) {
             if (state == FINE) t = fadd(t, tmu);
             else state = COARSE;
             continue;
         }
-        float den;
-        const float F = combined_value<MODE>(A, X, inv_s, den, true, t, lo, hi);
         if (state == FINE) {
             if (F <= 0.0f) {
                 state = WRONG;
@@ -270,8 +320,8 @@ __global__ void __launch_bounds__(256) raycast_combined_kernel(const CombinedArg
         for (int r = 0; r < 2; ++r) {
 #pragma unroll
             for (int i = 0; i < 3; ++i) X[i] = fadd(org[i], fmul(t, dir[i]));
-            float den;
-            const float F = combined_value<MODE>(A, X, inv_s, den, true, t, lo, hi);
+            float F, den;
+            combined_sample<MODE, false>(A, X, inv_s, t, lo, hi, F, den);
             t = fadd(t, fmul(F, tmu));
         }
 #pragma unroll
@@ -279,14 +329,15 @@ __global__ void __launch_bounds__(256) raycast_combined_kernel(const CombinedArg
         V = make_float4(X[0], X[1], X[2], 1.0f);
         float g[3];
         bool obs = true;
+        const unsigned near = submaps_near(A, X, inv_s);
 #pragma unroll 1
         for (int a = 0; a < 3; ++a) {
             float Xp[3] = {X[0], X[1], X[2]}, Xm[3] = {X[0], X[1], X[2]};
             Xp[a] = fadd(X[a], vs);
             Xm[a] = fsub(X[a], vs);
             float dp, dm;
-            const float fp = combined_value<MODE>(A, Xp, inv_s, dp);
-            const float fm = combined_value<MODE>(A, Xm, inv_s, dm);
+            const float fp = combined_value<MODE>(A, Xp, inv_s, near, dp);
+            const float fm = combined_value<MODE>(A, Xm, inv_s, near, dm);
             obs = obs && dp > 0.0f && dm > 0.0f;
             g[a] = fsub(fp, fm);
         }
