@@ -10,11 +10,15 @@
 //    J = (T p x N, N) give J J^T, J r, r^2 and a count.  The per-pixel
 //    arithmetic is float with each operation rounded on its own (built with
 //    -fmad=false), so the selection of pixels is the same on any IEEE
-//    machine; a thread accumulates its pixels (about four) in float and a
+//    machine; a thread accumulates its pixels (about eight) in float and a
 //    warp adds its lanes by a float shuffle tree (FP64 is a small fraction
 //    of the FP32 rate here); the CTA adds its warps in double and writes one
 //    partial row.  Each float sum is within 13 roundings of 2^-24 of the
-//    magnitude of its terms.
+//    magnitude of its terms.  Where a track does not converge, 19 steps make
+//    1e-4 of the pose out of the last bit of a sum, so the split of the
+//    pixels and the order of the sums are kept as they are (about eight pixels
+//    per thread at every level: more threads with fewer pixels at the coarse
+//    levels took the same time).
 //  * the CTA that finishes last adds the partial rows in a fixed order (the
 //    result does not depend on scheduling), then one of its warps solves
 //    H x = -g in double and applies the motion x = (omega, tau) on the world
@@ -29,16 +33,16 @@
 // so sums run with lanes as columns and few rows, and the solve keeps one
 // element of the symmetric system per lane.  640x480, three levels, 19 steps:
 // 800 us per track with one kernel for the sums and one for a serial solve by
-// a single thread (9 + 26 us per step), 330 us with this one (362 with IEEE divisions in
-// the solve and two divisions per pixel for its ray).
+// a single thread (9 + 26 us per step), 328 us with this one (362 with IEEE
+// divisions in the solve).
 #include "itm_ops.cuh"
 
 namespace itm {
 
 namespace {
 
-constexpr int kIcpThreads = 512, kIcpWarps = kIcpThreads / 32;
-constexpr int kBatch = 4;  // pixels of a thread per pass
+constexpr int kIcpThreads = 256, kIcpWarps = kIcpThreads / 32;
+constexpr int kBatch = 8;  // pixels of a thread per pass
 
 __global__ void __launch_bounds__(256) depth_halve_kernel(const float *__restrict__ in, int W, int H,
                                                           float *__restrict__ out)
@@ -78,7 +82,8 @@ __global__ void __launch_bounds__(32) track_begin_kernel(IcpState *st, Mat34 T)
 }
 
 // Sum over the warp of v[0 .. 31], value l ending in lane l: each stage halves
-// the values a lane holds (31 shuffles and adds instead of 5 per value).
+// the values a lane holds (31 shuffles and adds instead of 5 per value).  The
+// lanes 16, 8, 4, 2, 1 apart are added in that order.
 __device__ __forceinline__ float warp_sum32(float (&v)[32], int lane)
 {
 #pragma unroll
@@ -93,47 +98,36 @@ __device__ __forceinline__ float warp_sum32(float (&v)[32], int lane)
     return v[0];
 }
 
-// Lane l's column of the CTA's kIcpWarps rows in red, added in a fixed order:
-// complete in warp 0 (every thread of the CTA calls).
-__device__ __forceinline__ double column_sum(double (*red)[32], double x, int lane, int warp)
-{
-    red[warp][lane] = x;
-    __syncthreads();
-    if (warp < 4) {
-        x = red[4 * warp][lane];
-#pragma unroll
-        for (int k = 1; k < kIcpWarps / 4; ++k) x += red[4 * warp + k][lane];
-    }
-    __syncthreads();
-    if (warp < 4) red[warp][lane] = x;
-    __syncthreads();
-    return warp == 0 ? (red[0][lane] + red[1][lane]) + (red[2][lane] + red[3][lane]) : 0.0;
-}
-static_assert(kIcpWarps == 16, "column_sum adds four groups of four warps");
-
-// Columns of the n_part partial rows, added in a fixed order by the whole
-// CTA: lane l of warp 0 gets column l.
+// Columns of the n_part partial rows, added by the whole CTA: lane l of warp 0
+// gets column l.  Rows r, r + 32, ... are added in order for each r < 32, then
+// the 32 sums by halves (r with r + 16, 8, 4, 2, 1): the order in which a warp
+// with a row per lane adds them, here with a column per lane.
 __device__ __forceinline__ double row_sums(const double *__restrict__ partials, int n_part, double (*red)[32], int lane,
                                            int warp)
 {
-    double x = 0.0;
+    double x[4] = {0.0, 0.0, 0.0, 0.0};  // r = warp + 8 q
     if (lane < kIcpSums) {
-        // ten rows at a time (152 CTAs: one pass), their loads issued together
-        for (int b0 = warp; b0 < n_part; b0 += 10 * kIcpWarps) {
-            double r[10];
+        // 160 rows at a time, their loads issued together
+        for (int b0 = warp; b0 < n_part; b0 += 160) {
+            double v[20];
 #pragma unroll
-            for (int k = 0; k < 10; ++k) {
-                const int b = b0 + k * kIcpWarps;
-                r[k] = b < n_part ? __ldcg(&partials[(size_t)b * kIcpSums + lane]) : 0.0;
+            for (int k = 0; k < 20; ++k) {
+                const int b = b0 + 8 * k;
+                v[k] = b < n_part ? __ldcg(&partials[(size_t)b * kIcpSums + lane]) : 0.0;
             }
 #pragma unroll
-            for (int k = 0; k < 10; ++k)
-                if (b0 + k * kIcpWarps < n_part) x += r[k];  // uniform over the warp
+            for (int k = 0; k < 20; ++k)
+                if (b0 + 8 * k < n_part) x[k & 3] += v[k];  // uniform over the warp
         }
     }
     __syncthreads();  // red may still be read
-    return column_sum(red, x, lane, warp);
+    red[warp][lane] = (x[0] + x[2]) + (x[1] + x[3]);
+    __syncthreads();
+    if (warp != 0) return 0.0;
+    return ((red[0][lane] + red[4][lane]) + (red[2][lane] + red[6][lane])) +
+           ((red[1][lane] + red[5][lane]) + (red[3][lane] + red[7][lane]));
 }
+static_assert(kIcpWarps == 8, "row_sums adds eight warps' sums");
 
 // 1 / a to within an ulp of double: Newton's iteration y + y (1 - a y) from
 // the float reciprocal, whose error 2^-23 it squares twice (four FP64
@@ -240,35 +234,42 @@ __device__ __forceinline__ bool gauss_newton_warp(double x, IcpState *st, int la
 
 // Partial sums of CTA blockIdx.x: partials[b * kIcpSums + k].  The pose is
 // read from the tracker state st, and the CTA that finishes last takes the
-// step; or, with st null, from T_arg.  A thread takes pixels of one column, up
-// to kBatch of them rows rows apart (rows = ceil(H / batch): one division for
-// the column's ray, and the pixels of a warp still lie side by side): position
-// p of W x rows stands for pixels (p % W, p / W + b rows).  prefetch: the depth frame was
-// complete before the previous kernel of the stream began, so it is read
-// before the wait for that kernel.
+// step; or, with st null, from T_arg.  A thread takes the pixels p, p +
+// stride, ... in order, kBatch per pass: their depth loads, then their map
+// loads, are issued together.  prefetch: the depth frame was complete before
+// the previous kernel of the stream began, so the first pass's camera points
+// (which need no pose) are computed before the wait for that kernel, on the
+// SMs that its last CTA's solve leaves idle.
 __global__ void __launch_bounds__(kIcpThreads) icp_step_kernel(
     const float *__restrict__ depth, int W, int H, Intr in, IcpState *st, int level, Mat34 T_arg,
     const float4 *__restrict__ V, const float4 *__restrict__ N, Intr ref, Mat34 M, float dist_thresh,
-    double *__restrict__ partials, int rows, bool prefetch)
+    double *__restrict__ partials, bool prefetch)
 {
     __shared__ double red[kIcpWarps][32];
     __shared__ int is_last;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    // a pass's depth loads, then its map loads, are issued together
-    const int n_pos = W * rows, stride = gridDim.x * blockDim.x;
+    const int n_pix = W * H, stride = gridDim.x * blockDim.x;
     int p0 = blockIdx.x * blockDim.x + threadIdx.x;
-    float dk[kBatch];
-    auto read_depth = [&]() {
+    float pc[kBatch][3];  // camera points, z = 0: no depth
+    auto camera_points = [&]() {
 #pragma unroll
         for (int b = 0; b < kBatch; ++b) {
-            const int p = p0 + b * n_pos;  // row-major: b rows rows further down
-            dk[b] = p0 < n_pos && p < W * H ? __ldg(&depth[p]) : 0.0f;
+            const int p = p0 + b * stride;
+            const float d = p < n_pix ? __ldg(&depth[p]) : 0.0f;
+            pc[b][2] = d > 0.0f ? d : 0.0f;
+        }
+#pragma unroll
+        for (int b = 0; b < kBatch; ++b) {
+            const int p = p0 + b * stride;
+            const int u = p % W, v = p / W;
+            pc[b][0] = fmul(fdiv(fsub((float)u, in.cx), in.fx), pc[b][2]);
+            pc[b][1] = fmul(fdiv(fsub((float)v, in.cy), in.fy), pc[b][2]);
         }
     };
-    if (prefetch) read_depth();
+    if (prefetch) camera_points();
     grid_dep_wait();
     if (st && __ldcg(&st->done_level) == level) return;
-    if (!prefetch) read_depth();
+    if (!prefetch) camera_points();
     Mat34 T = T_arg;
     if (st) {
 #pragma unroll
@@ -279,29 +280,22 @@ __global__ void __launch_bounds__(kIcpThreads) icp_step_kernel(
 #pragma unroll
     for (int k = 0; k < 32; ++k) acc[k] = 0.0f;
     int count = 0;
-    while (p0 < n_pos) {
-        const int u = p0 % W, v = p0 / W;
-        const float rx = fdiv(fsub((float)u, in.cx), in.fx);
+    while (p0 < n_pix) {
         float pw[kBatch][3];
         int o[kBatch];
 #pragma unroll
         for (int b = 0; b < kBatch; ++b) {
             o[b] = -1;
-            const float d = dk[b];
-            if (d > 0.0f) {
-                const float pcx = fmul(rx, d);
-                const float pcy = fmul(fdiv(fsub((float)(v + b * rows), in.cy), in.fy), d);
-                float pr[3];
+            float pr[3];
 #pragma unroll
-                for (int r = 0; r < 3; ++r) pw[b][r] = row_apply(T.m + 4 * r, pcx, pcy, d);
+            for (int r = 0; r < 3; ++r) pw[b][r] = row_apply(T.m + 4 * r, pc[b][0], pc[b][1], pc[b][2]);
 #pragma unroll
-                for (int r = 0; r < 3; ++r) pr[r] = row_apply(M.m + 4 * r, pw[b][0], pw[b][1], pw[b][2]);
-                if (pr[2] > 0.0f) {
-                    const float ur = fadd(fdiv(fmul(ref.fx, pr[0]), pr[2]), ref.cx);
-                    const float vr = fadd(fdiv(fmul(ref.fy, pr[1]), pr[2]), ref.cy);
-                    if (ur >= 0.0f && ur <= (float)(ref.W - 1) && vr >= 0.0f && vr <= (float)(ref.H - 1))
-                        o[b] = (int)fadd(vr, 0.5f) * ref.W + (int)fadd(ur, 0.5f);
-                }
+            for (int r = 0; r < 3; ++r) pr[r] = row_apply(M.m + 4 * r, pw[b][0], pw[b][1], pw[b][2]);
+            if (pc[b][2] > 0.0f && pr[2] > 0.0f) {
+                const float ur = fadd(fdiv(fmul(ref.fx, pr[0]), pr[2]), ref.cx);
+                const float vr = fadd(fdiv(fmul(ref.fy, pr[1]), pr[2]), ref.cy);
+                if (ur >= 0.0f && ur <= (float)(ref.W - 1) && vr >= 0.0f && vr <= (float)(ref.H - 1))
+                    o[b] = (int)fadd(vr, 0.5f) * ref.W + (int)fadd(ur, 0.5f);
             }
         }
         float4 Vk[kBatch], Nk[kBatch];
@@ -314,8 +308,6 @@ __global__ void __launch_bounds__(kIcpThreads) icp_step_kernel(
                 Nk[b] = __ldg(&N[o[b]]);
             }
         }
-        p0 += stride;
-        read_depth();
 #pragma unroll
         for (int b = 0; b < kBatch; ++b) {
             if (o[b] < 0) continue;
@@ -328,24 +320,29 @@ __global__ void __launch_bounds__(kIcpThreads) icp_step_kernel(
             const float J[6] = {fsub(fmul(pw[b][1], Np.z), fmul(pw[b][2], Np.y)),
                                 fsub(fmul(pw[b][2], Np.x), fmul(pw[b][0], Np.z)),
                                 fsub(fmul(pw[b][0], Np.y), fmul(pw[b][1], Np.x)), Np.x, Np.y, Np.z};
-            // sums: one rounding per term (FMA)
             int k = 0;
 #pragma unroll
             for (int i = 0; i < 6; ++i)
 #pragma unroll
-                for (int j = i; j < 6; ++j, ++k) acc[k] = __fmaf_rn(J[i], J[j], acc[k]);
+                for (int j = i; j < 6; ++j, ++k) acc[k] = fadd(acc[k], fmul(J[i], J[j]));
 #pragma unroll
-            for (int i = 0; i < 6; ++i) acc[21 + i] = __fmaf_rn(J[i], res, acc[21 + i]);
-            acc[27] = __fmaf_rn(res, res, acc[27]);
+            for (int i = 0; i < 6; ++i) acc[21 + i] = fadd(acc[21 + i], fmul(J[i], res));
+            acc[27] = fadd(acc[27], fmul(res, res));
             ++count;
         }
+        p0 += kBatch * stride;
+        if (p0 < n_pix) camera_points();
     }
     // warps by float shuffle trees (the count is a whole number below 2^24:
     // exact), then the CTA's warp rows in double, in order
     static_assert(kIcpSums == 29, "28 sums and the count");
     acc[28] = (float)count;
-    const double x = column_sum(red, (double)warp_sum32(acc, lane), lane, warp);
+    red[warp][lane] = (double)warp_sum32(acc, lane);
+    __syncthreads();
     if (warp == 0) {
+        double x = 0.0;
+#pragma unroll
+        for (int w = 0; w < kIcpWarps; ++w) x += red[w][lane];
         if (lane < kIcpSums) {
             partials[(size_t)blockIdx.x * kIcpSums + lane] = x;
             __threadfence();
@@ -375,10 +372,9 @@ __global__ void __launch_bounds__(kIcpThreads) icp_sum_kernel(const double *__re
     if (warp == 0 && lane < kIcpSums) sums[lane] = x;
 }
 
-// Rows of a step's positions and its CTAs: one pixel per thread while there
-// are SMs for it (latency), then up to kBatch per thread and one CTA per SM
-// (few partial rows for the last CTA to add in FP64).
-int icp_shape(int W, int H, int &rows)
+// CTAs of a step: about eight pixels per thread, at most two CTAs per SM and
+// kIcpMaxPartials rows.  The split also fixes the order of the sums.
+int icp_grid(int n_pix)
 {
     static int sms = 0;
     if (!sms) {
@@ -387,13 +383,10 @@ int icp_shape(int W, int H, int &rows)
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (sms < 1) sms = 1;
     }
-    const int most = sms < kIcpMaxPartials ? sms : kIcpMaxPartials;
-    int batch = 1;
-    do
-        rows = (H + batch - 1) / batch;
-    while ((long long)W * rows > (long long)most * kIcpThreads && batch++ < kBatch);
-    const int g = (W * rows - 1) / kIcpThreads + 1;
-    return g < most ? g : most;
+    int g = (n_pix + 8 * kIcpThreads - 1) / (8 * kIcpThreads);
+    if (g > 2 * sms) g = 2 * sms;
+    if (g > kIcpMaxPartials) g = kIcpMaxPartials;
+    return g > 0 ? g : 1;
 }
 
 }  // namespace
@@ -410,11 +403,10 @@ cudaError_t launch_depth_halve(const float *in, int W, int H, float *out, cudaSt
 cudaError_t launch_icp_reduce(const float *depth, const Intr &in, const Mat34 &T_g, const float4 *V, const float4 *N,
                               const Intr &ref, const Mat34 &M_ref, float dist_thresh, double *work, cudaStream_t st)
 {
-    int rows = 0;
-    const int g = icp_shape(in.W, in.H, rows);
+    const int g = icp_grid(in.W * in.H);
     double *partials = work + kIcpSums;
     cudaError_t e = launch_pdl(icp_step_kernel, dim3(g), dim3(kIcpThreads), 0, st, depth, in.W, in.H, in,
-                               (IcpState *)nullptr, 0, T_g, V, N, ref, M_ref, dist_thresh, partials, rows, false);
+                               (IcpState *)nullptr, 0, T_g, V, N, ref, M_ref, dist_thresh, partials, false);
     if (e != cudaSuccess) return e;
     return launch_pdl(icp_sum_kernel, dim3(1), dim3(kIcpThreads), 0, st, (const double *)partials, g, work);
 }
@@ -469,12 +461,11 @@ cudaError_t launch_track(const float *depth, const Intr &in0, int levels, const 
     bool first = true;
     for (int l = levels - 1; l >= 0; --l) {
         if (iters[l] <= 0 || li[l].W < 1 || li[l].H < 1) continue;
-        int rows = 0;
-        const int g = icp_shape(li[l].W, li[l].H, rows);
+        const int g = icp_grid(li[l].W * li[l].H);
         for (int it = 0; it < iters[l]; ++it) {
             // the first step follows the pyramid's last kernel, which may have written its depth
             e = launch_pdl(icp_step_kernel, dim3(g), dim3(kIcpThreads), 0, st, lev[l], li[l].W, li[l].H, li[l], state,
-                           l + 1, Mat34{}, V, N, ref, M_ref, thresh[l], partials, rows, !first);
+                           l + 1, Mat34{}, V, N, ref, M_ref, thresh[l], partials, !first);
             if (e != cudaSuccess) return e;
             first = false;
         }
