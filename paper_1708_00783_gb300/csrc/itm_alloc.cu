@@ -1,23 +1,22 @@
 // Sec. 4.2 allocation on the GPU, in three launches per frame:
 //
 //  1. alloc_enumerate  one thread per pixel walks the blocks crossed by its
-//     segment d-mu .. d+mu (3D DDA).  The 32 lanes of a warp cover an 8x4
-//     pixel tile, so neighbouring rays emit mostly the same blocks: each step,
-//     __match_any_sync groups equal block keys and only one lane per group
-//     probes the hash.  A missing block claims its bucket's request word with
-//     one 64-bit CAS (the paper's per-entry allocation array, Sec. 4.2); the
-//     winner of a bucket appends the bucket to the request list, a block that
-//     finds its bucket claimed by another key goes to the overflow list
-//     (warp-aggregated appends, one atomic per warp).
+//     segment d-mu .. d+mu (3D DDA), a warp per 8x4 pixel tile.  The blocks
+//     are looked up in the brick table, those of a walk together.  A missing
+//     block claims its bucket's request word with one 64-bit CAS (the paper's
+//     per-entry allocation array, Sec. 4.2; equal keys of a warp grouped by
+//     __match_any_sync); the winner of a bucket appends the bucket to the
+//     request list, a block that finds its bucket claimed by another key goes
+//     to the overflow list (warp-aggregated appends).
 //  2. alloc_commit     one thread per requested bucket inserts its key
 //     (Sec. 3.3 insertion).  Each bucket's chain has exactly one writer, so
 //     chains are extended without locks; blocks and excess slots come from
 //     prepopulated free lists through warp-aggregated atomic counters (the
-//     paper's "atomic subtraction on a stack").  The CTA that finishes last
-//     then resolves the overflow list in rounds: look up, claim the bucket,
-//     let winners insert, repeat with the losers.  The paper leaves such
-//     intra-frame collisions for the next frame; resolving them makes the
-//     allocated set the complete union over all pixels.
+//     paper's "atomic subtraction on a stack").  In a frame with an overflow
+//     list the CTA that finishes last resolves it in rounds: look up, claim
+//     the bucket, let winners insert, repeat with the losers.  The paper
+//     leaves such intra-frame collisions for the next frame; resolving them
+//     makes the allocated set the complete union over all pixels.
 //  3. build_visible    every allocated block whose voxels can project into the
 //     image with z > 0 and lie within the frame's depth range + mu is
 //     appended to the visible list (Sec. 4.2, third part); eight lanes per
@@ -25,6 +24,12 @@
 //     the same pass also rasterises each block's search range.  It also enters
 //     the blocks this allocation handed out (a few dozen in a usual frame) in
 //     the brick table.
+//
+// The kernels run once through their code, so their length is dependent
+// accesses and code size: the insertion in the enumeration's warps took the
+// commit's launch out but cost a frame with thousands of new blocks more
+// (131 us against 38 + 38 in the 2 mm hall), in the visible pass it made that
+// pass 17 us instead of 8.
 //
 // Counts produced on the device are read by the next kernel from device
 // memory (persistent grid-stride loops), so no host synchronisation and no
@@ -42,66 +47,63 @@ __global__ void __launch_bounds__(256) alloc_enumerate_kernel(SceneDev s, const 
                                                               const uint16_t *__restrict__ raw,
                                                               float *__restrict__ depth_out)
 {
+    __shared__ int depth_max[8];
     const int cta = blockIdx.y * gridDim.x + blockIdx.x, ctas = gridDim.x * gridDim.y;
     grid_dep_wait();  // the previous raycast may still read the range tiles
+    FrameCounters *fc = &s.ctr->frame[__ldcg(&s.ctr->entered) & 1u];
+    if (cta == 0 && threadIdx.x == 0) frame_begin(s);
     for (int i = cta * blockDim.x + threadIdx.x; i < n_range_tiles; i += ctas * blockDim.x) {
         s.range_min[i] = 0xffffffffu;
         s.range_max[i] = 0u;
     }
-    enumerate_tile(s, depth, in, T, inv_b, blockIdx.x, blockIdx.y, raw, depth_out);
+    const int dm = enumerate_tile<4>(s, depth, in, T, inv_b, blockIdx.x, blockIdx.y, raw, depth_out, fc);
+    // one maximum per CTA: thousands on one word would wait for each other
+    if ((threadIdx.x & 31) == 0) depth_max[threadIdx.x >> 5] = dm;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int m = 0;
+        for (int w = 0; w < 8; ++w) m = max(m, depth_max[w]);
+        if (m > 0) atomicMax(&fc->depth_max_bits, m);
+    }
     grid_dep_launch();
 }
 
-// The last CTA to finish its requests then resolves the overflow list (its
-// inserts are visible through the fences before the completion count).
 __global__ void __launch_bounds__(256) alloc_commit_kernel(SceneDev s)
 {
     __shared__ int is_last, remaining;
     grid_dep_wait();
-    const int n = min(__ldcg(&s.ctr->n_req), s.nb);
+    FrameCounters *fc = frame_set(s);
+    const int n = min(__ldcg(&fc->n_req), s.nb), n_overflow = __ldcg(&fc->n_overflow);
     const int stride = gridDim.x * blockDim.x;
-    for (int i0 = blockIdx.x * blockDim.x; i0 < n; i0 += stride) {
-        const int i = i0 + threadIdx.x;
-        if (i < n) commit_request(s, i);
-    }
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) is_last = atomicAdd(&s.ctr->commit_done, 1) == (int)gridDim.x - 1;
-    __syncthreads();
-    if (is_last) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) commit_request(s, i);
+    if (blockIdx.x == 0 && threadIdx.x == 0) frame_end(s);
+    if (n_overflow > 0) {
         __threadfence();
-        overflow_scene(s, remaining);
+        __syncthreads();
+        if (threadIdx.x == 0) is_last = atomicAdd(&fc->done, 1) == (int)gridDim.x - 1;
+        __syncthreads();
+        if (is_last) {
+            __threadfence();
+            overflow_scene(s, n_overflow, remaining);
+        }
     }
     grid_dep_launch();
 }
 
-__global__ void __launch_bounds__(256) build_visible_kernel(SceneDev s, Mat34 M, Intr in)
+// RANGE: also fill the search range of a raycast from this pose (zc, tiles).
+// The loop is uniform per CTA; a warp's four groups of eight lanes hold a
+// block each.
+template <bool RANGE>
+__global__ void __launch_bounds__(256) build_visible_kernel(SceneDev s, Mat34 M, Intr in, float zc, int tiles_x,
+                                                            int tiles_y)
 {
     grid_dep_wait();
-    const int n = min(__ldcg(&s.ctr->block_head), s.nv);
-    const float zfar = visible_zfar(s);
-    const int brick_from = __ldcg(&s.ctr->brick_from);
+    const int n = min(__ldcg(&s.ctr->block_head), s.nv), head_before = __ldcg(&s.ctr->head_before);
+    const float zfar = visible_zfar(s, frame_set(s));
     const int groups = gridDim.x * (blockDim.x >> 3);
     for (int g0 = blockIdx.x * (blockDim.x >> 3); g0 < n; g0 += groups) {
         const int i = g0 + (threadIdx.x >> 3);
-        visible_8<false>(s, M, in, zfar, brick_from, i < n, i, 0.0f, 1, 1);
-    }
-    grid_dep_launch();
-}
-
-// The same, also filling the search range of a raycast from this pose (the
-// loop is uniform per CTA so every warp reaches the rasterisation together).
-__global__ void __launch_bounds__(256) build_visible_range_kernel(SceneDev s, Mat34 M, Intr in, float zc,
-                                                                  int tiles_x, int tiles_y)
-{
-    grid_dep_wait();
-    const int n = min(__ldcg(&s.ctr->block_head), s.nv);
-    const float zfar = visible_zfar(s);
-    const int brick_from = __ldcg(&s.ctr->brick_from);
-    const int groups = gridDim.x * (blockDim.x >> 3);
-    for (int g0 = blockIdx.x * (blockDim.x >> 3); g0 < n; g0 += groups) {
-        const int i = g0 + (threadIdx.x >> 3);
-        visible_8<true>(s, M, in, zfar, brick_from, i < n, i, zc, tiles_x, tiles_y);
+        visible_8<RANGE>(s, M, in, zfar, head_before, i < n, i, zc, tiles_x, tiles_y);
     }
     grid_dep_launch();
 }
@@ -131,30 +133,26 @@ int persistent_grid(int threads, const void *kernel)
 cudaError_t launch_allocate(const SceneDev &s, const float *depth, const Intr &in, const Mat34 &T_wc,
                             const Mat34 &M_d, bool with_range, cudaStream_t st, const uint16_t *raw)
 {
-    static_assert(kFrameCountersOffset % 4 == 0 && kFrameCountersBytes % 4 == 0, "word-aligned frame counters");
-    cudaError_t e = launch_pdl(alloc_begin_kernel, dim3(1), dim3(32), 0, st, s.ctr);
-    if (e != cudaSuccess) return e;
     const float inv_b = (float)(1.0 / (8.0 * (double)s.voxel_size));
     dim3 grid((in.W + 31) / 32, (in.H + 7) / 8);
     const int n_range_tiles = with_range ? ((in.W + 7) / 8) * ((in.H + 3) / 4) : 0;
     // with raw, depth is the output of the frame's conversion
-    e = launch_pdl(alloc_enumerate_kernel, grid, dim3(256), 0, st, s, raw ? nullptr : depth, in, T_wc, inv_b,
+    cudaError_t e = launch_pdl(alloc_enumerate_kernel, grid, dim3(256), 0, st, s, raw ? nullptr : depth, in, T_wc, inv_b,
                    n_range_tiles, raw, raw ? const_cast<float *>(depth) : nullptr);
     if (e != cudaSuccess) return e;
     static int g_commit = 0, g_visible = 0, g_visrange = 0;
-    // one CTA per SM: a frame's requests (usually a few thousand) fit in one
-    // pass, and fewer CTAs pay the completion count's fences
+    // one CTA per SM: a frame's requests (usually a few thousand) fit in one pass
     if (!g_commit) g_commit = sm_count();
-    if (!g_visible) g_visible = persistent_grid(256, (const void *)build_visible_kernel);
-    if (!g_visrange) g_visrange = persistent_grid(256, (const void *)build_visible_range_kernel);
+    if (!g_visible) g_visible = persistent_grid(256, (const void *)build_visible_kernel<false>);
+    if (!g_visrange) g_visrange = persistent_grid(256, (const void *)build_visible_kernel<true>);
     e = launch_pdl(alloc_commit_kernel, dim3(g_commit), dim3(256), 0, st, s);
     if (e != cudaSuccess) return e;
     if (with_range) {
         const int tx = (in.W + 7) / 8, ty = (in.H + 3) / 4;
-        e = launch_pdl(build_visible_range_kernel, dim3(g_visrange), dim3(256), 0, st, s, M_d, in, s.z_min - 1e-3f,
+        e = launch_pdl(build_visible_kernel<true>, dim3(g_visrange), dim3(256), 0, st, s, M_d, in, s.z_min - 1e-3f,
                        tx, ty);
     } else {
-        e = launch_pdl(build_visible_kernel, dim3(g_visible), dim3(256), 0, st, s, M_d, in);
+        e = launch_pdl(build_visible_kernel<false>, dim3(g_visible), dim3(256), 0, st, s, M_d, in, 0.0f, 1, 1);
     }
     return e;
 }

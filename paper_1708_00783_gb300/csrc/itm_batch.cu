@@ -97,9 +97,7 @@ __global__ void __launch_bounds__(256) batch_begin_kernel(const ItemDev *__restr
     const int n = head->n;
     if ((int)blockIdx.x >= n) return;
     const ItemDev &it = items[blockIdx.x];
-    if (threadIdx.x < kFrameCountersBytes / 4)
-        reinterpret_cast<int *>(reinterpret_cast<char *>(it.s.ctr) + kFrameCountersOffset)[threadIdx.x] = 0;
-    if (threadIdx.x == 31) it.s.ctr->brick_from = it.s.ctr->block_head;
+    if (threadIdx.x == 0) frame_begin(it.s);
     const int tiles = it.rtiles_x * it.rtiles_y;
     for (int i = threadIdx.x; i < tiles; i += blockDim.x) {
         it.s.range_min[i] = 0xffffffffu;
@@ -107,7 +105,7 @@ __global__ void __launch_bounds__(256) batch_begin_kernel(const ItemDev *__restr
     }
 }
 
-__global__ void __launch_bounds__(256) batch_enumerate_kernel(const ItemDev *__restrict__ items, const BatchHead *head,
+__global__ void __launch_bounds__(256, 8) batch_enumerate_kernel(const ItemDev *__restrict__ items, const BatchHead *head,
                                                                 bool scatter)
 {
     __shared__ int begin[kMaxItems + 1];
@@ -119,7 +117,11 @@ __global__ void __launch_bounds__(256) batch_enumerate_kernel(const ItemDev *__r
         const int k = find_item(begin, n, vt);
         const ItemDev &it = items[k];
         const int local = vt - begin[k];
-        enumerate_tile(it.s, it.depth, it.in, it.T, it.inv_b, local % it.cta_tiles_x, local / it.cta_tiles_x);
+        FrameCounters *fc = frame_set(it.s);
+        const int known = __ldcg(&fc->depth_max_bits);
+        const int dm = enumerate_tile<1>(it.s, it.depth, it.in, it.T, it.inv_b, local % it.cta_tiles_x,
+                                      local / it.cta_tiles_x, nullptr, nullptr, fc);
+        if ((threadIdx.x & 31) == 0 && dm > known) atomicMax(&fc->depth_max_bits, dm);
     }
 }
 
@@ -128,7 +130,7 @@ __global__ void __launch_bounds__(256) batch_commit_kernel(const ItemDev *__rest
     __shared__ int prefix[kMaxItems + 1];
     const int n = head->n;
     const int total = cta_prefix(items, n, prefix, [](const ItemDev &it) {
-        return min(__ldcg(&it.s.ctr->n_req), it.s.nb);
+        return min(__ldcg(&frame_set(it.s)->n_req), it.s.nb);
     });
     for (int i0 = blockIdx.x * blockDim.x; i0 < total; i0 += gridDim.x * blockDim.x) {
         const int i = i0 + threadIdx.x;
@@ -143,7 +145,9 @@ __global__ void __launch_bounds__(kOvfThreads) batch_overflow_kernel(const ItemD
 {
     __shared__ int remaining;
     if ((int)blockIdx.x >= head->n) return;
-    overflow_scene(items[blockIdx.x].s, remaining);
+    const SceneDev &s = items[blockIdx.x].s;
+    overflow_scene(s, __ldcg(&frame_set(s)->n_overflow), remaining);
+    if (threadIdx.x == 0) frame_end(s);
 }
 
 __global__ void __launch_bounds__(256) batch_visible_kernel(const ItemDev *__restrict__ items, const BatchHead *head)
@@ -158,7 +162,7 @@ __global__ void __launch_bounds__(256) batch_visible_kernel(const ItemDev *__res
         if (i >= total) continue;
         const int k = find_item(prefix, n, i);
         const ItemDev &it = items[k];
-        visible_block(it.s, it.M, it.in, visible_zfar(it.s), i - prefix[k]);
+        visible_block(it.s, it.M, it.in, visible_zfar(it.s, frame_set(it.s)), i - prefix[k]);
     }
 }
 

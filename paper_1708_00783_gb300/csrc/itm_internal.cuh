@@ -61,26 +61,32 @@ struct __align__(16) Entry {
     int32_t ptr;     // >= 0 block index; -1 swapped out; < -1 unallocated (Sec. 3.2)
 };
 
+// Counts of one allocation.
+struct FrameCounters {
+    int32_t n_req;          // buckets requested
+    int32_t n_overflow;     // requests that lost their bucket
+    int32_t depth_max_bits; // largest valid depth (float bits, >= 0)
+    int32_t done;           // CTAs of the visible-list pass that finished (frames with an overflow)
+};
+
+// Two sets of frame counts take turns, so that no launch in front of an
+// allocation has to clear them.  The enumeration reads `entered` and counts in
+// set entered & 1; it writes `begun`, from which the passes after it know the
+// set (frame_set); the first of them to follow clears the other set and
+// writes `entered`.  Neither word is read by a kernel that writes it.
 struct Counters {
     uint32_t status;
     int32_t block_head;     // blocks handed out (may run past nv when the array is full)
     int32_t excess_head;    // excess slots handed out
-    int32_t n_req;          // per-frame: buckets requested
-    int32_t n_overflow;     // per-frame: requests that lost their bucket
-    int32_t n_visible;      // per-frame: visible blocks
-    int32_t depth_max_bits; // per-frame: largest valid depth (float bits, >= 0)
-    int32_t commit_done;    // per-frame: CTAs of the commit kernel that finished
+    int32_t n_visible;      // visible blocks
+    int32_t head_before;    // blocks handed out before the last allocation
+    uint32_t begun, entered;  // allocations whose enumeration / whose commit has run
+    FrameCounters frame[2];
     unsigned long long updated;  // cumulative voxel updates
     unsigned long long visited;  // cumulative voxels visited by integration
     unsigned long long frames;   // cumulative integrated frames
     unsigned long long mesh_tris;  // per-mesh: triangles found
-    int32_t brick_from;  // per-frame: blocks handed out before it (they are in the brick table)
 };
-
-// Offset and size of the per-frame counters cleared at the start of allocation.
-constexpr size_t kFrameCountersOffset = 12;  // n_req
-constexpr size_t kFrameCountersBytes = 20;   // n_req .. commit_done
-
 
 struct SceneDev {
     Entry *entries;
@@ -227,9 +233,9 @@ __device__ __forceinline__ int lookup_cg(const SceneDev &s, int bx, int by, int 
 // the room; cells with a tag of their own instead of the place's owner took a
 // fifth more instructions.)
 //
-// Blocks enter in the visible pass after the allocation that handed them out
-// (and after an import), and leave in the swap-out; the kernels that change
-// the table and those that read it never run at the same time.
+// Blocks enter in the pass of the allocation that hands them out (and after an
+// import), and leave in the swap-out; the kernels that change the table and
+// those that read it never run at the same time.
 constexpr int kBrickSide = 9;      // blocks along a brick's edge with the one further
 constexpr int kBrickCells = 736;   // 9^3 cells, rounded up to whole 32-byte sectors
 constexpr int kBrickMin = 4096;    // smallest number of places (12 MB)
@@ -271,15 +277,27 @@ static __device__ __noinline__ int lookup_chain(const SceneDev &s, int bx, int b
     return lookup_ro(s, bx, by, bz);
 }
 
-// The block index at (bx, by, bz), or -1.
+// The block index at (bx, by, bz), or -1; in two parts, so that the loads of
+// several blocks can be issued together.
+struct BrickCell {
+    unsigned long long own;
+    int ptr;
+};
+__device__ __forceinline__ BrickCell brick_load(const SceneDev &s, int bx, int by, int bz)
+{
+    const uint32_t place = brick_place(bx >> 3, by >> 3, bz >> 3, s.brick_mask);
+    return {__ldg(&s.brick_owner[place]),
+            __ldg(&s.brick_cell[(size_t)place * kBrickCells + brick_local(bx & 7, by & 7, bz & 7)])};
+}
+__device__ __forceinline__ int brick_answer(const SceneDev &s, int bx, int by, int bz, const BrickCell &c)
+{
+    if ((c.own & ~kBrickShared) == brick_key(bx >> 3, by >> 3, bz >> 3))
+        return ITM_IN_BOUNDS(s, c.ptr < s.nv) ? c.ptr : -1;
+    return c.own & kBrickShared ? lookup_chain(s, bx, by, bz) : -1;
+}
 __device__ __forceinline__ int brick_find(const SceneDev &s, int bx, int by, int bz)
 {
-    const int X = bx >> 3, Y = by >> 3, Z = bz >> 3;
-    const uint32_t place = brick_place(X, Y, Z, s.brick_mask);
-    const unsigned long long own = __ldg(&s.brick_owner[place]), key = brick_key(X, Y, Z);
-    const int p = __ldg(&s.brick_cell[(size_t)place * kBrickCells + brick_local(bx & 7, by & 7, bz & 7)]);
-    if ((own & ~kBrickShared) == key) return ITM_IN_BOUNDS(s, p < s.nv) ? p : -1;
-    return own & kBrickShared ? lookup_chain(s, bx, by, bz) : -1;
+    return brick_answer(s, bx, by, bz, brick_load(s, bx, by, bz));
 }
 
 // The blocks of the 2x2x2 neighbourhood of block (bx, by, bz) towards +x, +y,
@@ -437,18 +455,6 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
 }
 
 namespace {
-// The start of an allocation: its counters cleared, the blocks handed out so
-// far noted (they are in the brick table).  A kernel of the chain and not a
-// memset, which would break it.
-__global__ void __launch_bounds__(32) alloc_begin_kernel(Counters *ctr)
-{
-    grid_dep_wait();
-    if (threadIdx.x < kFrameCountersBytes / 4)
-        reinterpret_cast<int32_t *>(reinterpret_cast<char *>(ctr) + kFrameCountersOffset)[threadIdx.x] = 0;
-    if (threadIdx.x == 31) ctr->brick_from = ctr->block_head;
-    grid_dep_launch();
-}
-
 // Zeroes n 32-bit words at p after the previous kernel (a launch_pdl stand-in
 // for cudaMemsetAsync, which would break the chain of dependent launches).
 __global__ void __launch_bounds__(32) zero_words_kernel(int32_t *p, int n)

@@ -601,8 +601,8 @@ int itm_scene_stats(itm_scene *sc, itm_stats *out)
     out->allocated_blocks = c.block_head < sc->d.nv ? c.block_head : sc->d.nv;
     out->excess_used = c.excess_head < sc->d.ne ? c.excess_head : sc->d.ne;
     out->visible_blocks = c.n_visible;
-    out->last_requests = c.n_req;
-    out->last_overflow = c.n_overflow;
+    out->last_requests = c.frame[(c.begun - 1u) & 1u].n_req;
+    out->last_overflow = c.frame[(c.begun - 1u) & 1u].n_overflow;
     out->updated_voxels = c.updated;
     out->visited_voxels = c.visited;
     out->frames = c.frames;
@@ -781,7 +781,6 @@ int itm_scene_import(itm_scene *sc, const int16_t *coords_host, const float *sdf
         memset(&c, 0, sizeof(c));
         c.block_head = n;
         c.excess_head = used_excess;
-        c.brick_from = n;
         e = cudaMemcpy(d.ctr, &c, sizeof(c), cudaMemcpyHostToDevice);
     }
     if (e == cudaSuccess) e = launch_brick_fill(d, n, 0);
