@@ -34,12 +34,8 @@ constexpr int kBlockVoxels = 512;
 // largest image whose raycast uses the search-range tiles (8x4 pixels each)
 constexpr int kRangeMaxW = 4096, kRangeMaxH = 4096;
 constexpr int kRangeMaxTiles = (kRangeMaxW / 8) * (kRangeMaxH / 4);
-// Raycast tiles are handed out by cost class (march iterations / 8, heaviest
-// first) as measured by the previous raycast, for images of at most
-// kOrderMaxTiles tiles.
-constexpr int kOrderMaxTiles = 1 << 16;
-constexpr int kTileClasses = 16;
-constexpr int kTileHdrInts = 32;  // per side: next, counts[kTileClasses], padding
+// rays that the raycast's slow list has room for (larger images march every ray in the first phase)
+constexpr int kSlowMax = 1 << 21;
 constexpr int kCombinedMax = ITM_COMBINED_MAX;
 constexpr int kIcpSums = ITM_ICP_SUMS;
 constexpr int kIcpWorkDoubles = ITM_ICP_WORK_DOUBLES;
@@ -88,6 +84,16 @@ struct Counters {
     unsigned long long mesh_tris;  // per-mesh: triangles found
 };
 
+// Counts of one raycast: its next tile, its slow rays.  Two sets take turns as
+// in Counters: the first phase reads `entered` and writes `begun`, the second
+// reads `begun`, clears the other set and writes `entered`.
+struct RayCounters {
+    uint32_t begun, entered;
+    struct {
+        int32_t next, n_slow;
+    } set[2];
+};
+
 struct SceneDev {
     Entry *entries;
     unsigned long long *req;
@@ -107,11 +113,8 @@ struct SceneDev {
     uint32_t brick_mask;              // places - 1
     uint32_t *range_min;  // per 8x4 tile: nearest / farthest depth (float bits) of covering blocks
     uint32_t *range_max;
-    // raycast tile queues, two sides (one written by a raycast, the other
-    // read): per side a header {next tile, count of each cost class} and per
-    // class a list of up to kOrderMaxTiles tiles
-    int32_t *tile_q_hdr;
-    int32_t *tile_q_list;
+    RayCounters *ray_ctr;
+    int32_t *slow_list;  // kSlowMax pixels: rays not through with the raycast's first phase
     // Sec. 5 swapping: null while swapping is off
     uint8_t *swap_state;
     int32_t *touch;
@@ -454,17 +457,6 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
-namespace {
-// Zeroes n 32-bit words at p after the previous kernel (a launch_pdl stand-in
-// for cudaMemsetAsync, which would break the chain of dependent launches).
-__global__ void __launch_bounds__(32) zero_words_kernel(int32_t *p, int n)
-{
-    grid_dep_wait();
-    for (int i = threadIdx.x; i < n; i += blockDim.x) p[i] = 0;
-    grid_dep_launch();
-}
-}  // namespace
-
 // ------------------------------------------------ IEEE round-to-nearest ops
 // Every operation that decides an integer (which block, which pixel, whether
 // a voxel is updated) is written with these so that no multiply-add is fused.
@@ -511,11 +503,6 @@ struct itm_scene {
     long long range_epoch;
     float range_pose[16];
     itm_intrinsics range_intr;
-    // the tile queues of side 1 - (order_side & 1) hold every tile of a
-    // tiles_x x tiles_y image ({0, 0}: none yet); the next raycast writes side
-    // order_side & 1, whose header is already clear when bit 1 is set
-    int order_dims[2];
-    int order_side;
     // the visible list's interior flags were computed for vis_pose /
     // vis_intr (vis_ok: by the last allocation, with no block moved or freed
     // since)
@@ -562,7 +549,7 @@ cudaError_t launch_allocate(const SceneDev &s, const float *depth, const Intr &i
 cudaError_t launch_integrate(const SceneDev &s, const float *depth, const float *wpx, const Intr &in,
                              const Mat34 &M_d, bool interior_ok, cudaStream_t st);
 cudaError_t launch_raycast(const SceneDev &s, const Intr &in, const Mat34 &T_wc, const Mat34 &M_d, float4 *vtx,
-                           float4 *nrm, bool range_ready, int order_dims[2], int &order_side, cudaStream_t st);
+                           float4 *nrm, bool range_ready, cudaStream_t st);
 cudaError_t launch_raycast_range(const SceneDev &s, const Intr &in, const Mat34 &M_d, uint32_t *rmin, uint32_t *rmax,
                                  cudaStream_t st);
 bool range_fits(const Intr &in);

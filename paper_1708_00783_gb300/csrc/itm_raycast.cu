@@ -66,93 +66,85 @@ __global__ void __launch_bounds__(256) range_kernel(SceneDev s, Mat34 M, Intr in
 
 // Persistent raycast, first phase (the march): each warp takes the next 8x4
 // tile from a device counter until none is left, so warps that finish early
-// pick up more work instead of idling behind the slowest tiles of a fixed
-// grid.  raycast_finish_kernel then refines the hits and takes their normals
-// (two kernels with smaller code each measured faster than the one that did
-// both).  With use_order the tiles
-// are handed out from the queues of the previous raycast, heaviest cost class
-// first (longest processing time first), so the expensive tiles do not start
-// last.  With write_order each finished tile is appended to the queue of its
-// cost class for the next raycast.  hdr_w[0] is this raycast's tile counter.
+// pick up more work.  Rays that are not through after a while go to the slow
+// list (room: as many as the second phase takes at once; 0: none).
+//
+// Most rays end within 6 to 10 iterations, but those that skim a wall or leave
+// the mapped part take 80 (room) to 190 (2 mm hall), each two dependent memory
+// accesses long (0.7 us): marched to their end in their own tiles they were
+// most of the raycast (56 to 80 us of it in the room, 28 to 36 us at 160x120),
+// with the chip idle.  Now they continue in the second kernel with four lanes a
+// ray (march_slow), beside the finish of the others.
 template <int MODE>
-__global__ void __launch_bounds__(256, 4) raycast_dynamic_kernel(SceneDev s, Intr in, Mat34 T, float4 *__restrict__ vtx,
-                                                              float4 *__restrict__ nrm, int max_iter, float tB_m,
-                                                              float inv_sv, const uint32_t *__restrict__ rmin,
-                                                              const uint32_t *__restrict__ rmax, int tiles_x,
-                                                              int n_tiles, int32_t *__restrict__ hdr_w,
-                                                              int32_t *__restrict__ list_w,
-                                                              const int32_t *__restrict__ hdr_r,
-                                                              const int32_t *__restrict__ list_r, bool use_order,
-                                                              bool write_order)
+__global__ void __launch_bounds__(256, 4) raycast_march_kernel(SceneDev s, Intr in, Mat34 T, float4 *__restrict__ vtx,
+                                                               int max_iter, float tB_m, float inv_sv,
+                                                               const uint32_t *__restrict__ rmin,
+                                                               const uint32_t *__restrict__ rmax, int tiles_x,
+                                                               int n_tiles, int room)
 {
-    // first position of each class slot k (class kTileClasses - 1 - k)
-    __shared__ int first[kTileClasses + 1];
     const int lane = threadIdx.x & 31;
     grid_dep_wait();
-    if (use_order) {
-        if (threadIdx.x == 0) {
-            int acc = 0;
-            for (int k = 0; k < kTileClasses; ++k) {
-                first[k] = acc;
-                acc += __ldg(&hdr_r[1 + kTileClasses - 1 - k]);
-            }
-            first[kTileClasses] = acc;
-        }
-        __syncthreads();
-        // queues that do not hold every tile once (cannot happen when the
-        // previous raycast covered the same tiles) fall back to raster order
-        use_order = first[kTileClasses] == n_tiles;
-    }
+    const uint32_t entered = __ldcg(&s.ray_ctr->entered);
+    auto *c = &s.ray_ctr->set[entered & 1u];
+    if (blockIdx.x == 0 && threadIdx.x == 0) s.ray_ctr->begun = entered + 1u;
     for (;;) {
         int t = 0;
-        if (lane == 0) t = atomicAdd(&hdr_w[0], 1);
+        if (lane == 0) t = atomicAdd(&c->next, 1);
         t = __shfl_sync(kFull, t, 0);
-        if (t >= n_tiles) {
-            grid_dep_launch();
-            return;
-        }
-        int tile = t;
-        if (use_order) {
-            int k = 0;
-            while (k < kTileClasses - 1 && first[k + 1] <= t) ++k;
-            tile = __ldg(&list_r[(size_t)(kTileClasses - 1 - k) * kOrderMaxTiles + (t - first[k])]);
-            if ((unsigned)tile >= (unsigned)n_tiles) tile = t;
-        }
-        const int cost = raycast_warp_tile<MODE, true, 1>(s, in, T, vtx, nrm, max_iter, tB_m, inv_sv, rmin, rmax,
-                                                          tiles_x, tile % tiles_x, tile / tiles_x);
-        if (write_order && lane == 0) {
-            const int c = min(cost >> 3, kTileClasses - 1);
-            const int p = atomicAdd(&hdr_w[1 + c], 1);
-            list_w[(size_t)c * kOrderMaxTiles + p] = tile;
-        }
+        if (t >= n_tiles) break;
+        raycast_march_tile<MODE>(s, in, T, vtx, max_iter, tB_m, inv_sv, rmin, rmax, tiles_x, t % tiles_x, t / tiles_x,
+                                 room > 0 ? &c->n_slow : nullptr, room);
+    }
+    grid_dep_launch();
+}
+
+// Second phase: refinement, hit point and normal of the rays that ended (two
+// kernels with smaller code each measured faster than the one that did both),
+// beside the slow rays to their end.  The first slow_ctas CTAs take the groups
+// of the slow list, the first warp of each before the second, ...: of eight
+// rays while there are warps for them, of up to 32 beyond that, where filled
+// finish passes count for more than latency.
+template <int MODE>
+__global__ void __launch_bounds__(256, 4) raycast_finish_kernel(SceneDev s, Intr in, Mat34 T, float4 *vtx, float4 *nrm,
+                                                                int max_iter, float tB_m, float inv_sv,
+                                                                const uint32_t *__restrict__ rmin,
+                                                                const uint32_t *__restrict__ rmax, int tiles_x,
+                                                                int tiles, int slow_ctas)
+{
+    grid_dep_wait();
+    RayCounters *c = s.ray_ctr;
+    const uint32_t begun = __ldcg(&c->begun);
+    const int warp = threadIdx.x >> 5, cta = (int)blockIdx.x - slow_ctas;
+    if (cta == 0 && threadIdx.x == 0) {
+        // the next raycast's set; nothing reads it before that
+        c->set[begun & 1u].next = c->set[begun & 1u].n_slow = 0;
+        c->entered = begun;
+    }
+    const int n_slow = cta < 0 ? min(__ldcg(&c->set[(begun - 1u) & 1u].n_slow), kSlowMax) : 0;
+    const int rounds = min((n_slow - 1) / (64 * slow_ctas) + 1, 4);
+    for (int g = cta < 0 ? (int)blockIdx.x + slow_ctas * warp : cta * 8 + warp;
+         cta < 0 ? g * 8 * rounds < n_slow : g < tiles; g += cta < 0 ? 8 * slow_ctas : tiles) {
+        const EndedRay e = cta < 0 ? raycast_slow_rays<MODE>(s, in, T, vtx, max_iter, tB_m, inv_sv, rmin, rmax, tiles_x,
+                                                             g * 8 * rounds, rounds, n_slow)
+                                   : raycast_tile_rays(in, vtx, g % tiles_x, g / tiles_x);
+        finish_ray<MODE>(s, in, T, tB_m, inv_sv, e, vtx, nrm);
     }
 }
 
-// second phase of the split raycast: refinement, hit point and normal of the
-// pixels whose march (raycast_dynamic_kernel) ended behind the surface.
-// hdr_clear (or null): the tile-queue header the march read, cleared for the
-// next raycast, which writes that side (so it needs no clearing launch).
+// Without a search range (images beyond the range tiles): the whole raycast
+// of one pixel per thread.
 template <int MODE>
-__global__ void __launch_bounds__(256, 4) raycast_finish_kernel(SceneDev s, Intr in, Mat34 T, float4 *__restrict__ vtx,
-                                                             float4 *__restrict__ nrm, int max_iter, float tB_m,
-                                                             float inv_sv, int32_t *__restrict__ hdr_clear)
-{
-    grid_dep_wait();
-    if (hdr_clear && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < kTileHdrInts) hdr_clear[threadIdx.x] = 0;
-    const int warp = threadIdx.x >> 5;
-    const int tix = blockIdx.x * 4 + (warp & 3), tiy = blockIdx.y * 2 + (warp >> 2);
-    if (tix >= (in.W + 7) / 8 || tiy >= (in.H + 3) / 4) return;
-    raycast_warp_tile<MODE, false, 2>(s, in, T, vtx, nrm, max_iter, tB_m, inv_sv, nullptr, nullptr, 0, tix, tiy);
-}
-
-template <int MODE, bool RANGE>
 __global__ void __launch_bounds__(256) raycast_kernel(SceneDev s, Intr in, Mat34 T, float4 *__restrict__ vtx,
-                                                      float4 *__restrict__ nrm, int max_iter, float tB_m,
-                                                      float inv_sv, const uint32_t *__restrict__ rmin,
-                                                      const uint32_t *__restrict__ rmax, int tiles_x, int tiles_y)
+                                                      float4 *__restrict__ nrm, int max_iter, float tB_m, float inv_sv)
 {
-    raycast_tile<MODE, RANGE>(s, in, T, vtx, nrm, max_iter, tB_m, inv_sv, rmin, rmax, tiles_x, tiles_y, blockIdx.x,
-                              blockIdx.y);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int u = (blockIdx.x * 4 + (warp & 3)) * 8 + (lane & 7), v = (blockIdx.y * 2 + (warp >> 2)) * 4 + (lane >> 3);
+    const bool inside = u < in.W && v < in.H;
+    const Ray r = make_ray(s, in, T, tB_m, u, v);
+    float t;
+    int state, it;
+    march_warp<MODE, false>(s, r, inside, max_iter, inv_sv, nullptr, nullptr, 0, nullptr, 0, t, state, it);
+    if (inside) finish_pixel<MODE>(s, r, state == BEHIND, t, inv_sv, (size_t)v * in.W + u, vtx, nrm);
 }
 
 int range_grid()
@@ -184,79 +176,54 @@ cudaError_t launch_raycast_range(const SceneDev &s, const Intr &in, const Mat34 
 }
 
 cudaError_t launch_raycast(const SceneDev &s, const Intr &in, const Mat34 &T_wc, const Mat34 &M_d, float4 *vtx,
-                           float4 *nrm, bool range_ready, int order_dims[2], int &order_side, cudaStream_t st)
+                           float4 *nrm, bool range_ready, cudaStream_t st)
 {
     // host-side constants with the same float operations as the oracle
     volatile float span = s.z_max - s.z_min;
     volatile float four_span = 4.0f * span;
     volatile float ratio = four_span / s.voxel_size;
     const int max_iter = (int)ratio + 64;
-    volatile float tB_m = 8.0f * s.voxel_size;
+    volatile float tB_v = 8.0f * s.voxel_size;
+    const float tB_m = tB_v;
     const float inv_sv = (float)(1.0 / (double)s.voxel_size);  // voxel coordinates: p * (1/s), 1/s rounded once
     dim3 grid((in.W + 31) / 32, (in.H + 7) / 8);
     const int tx = (in.W + 7) / 8, ty = (in.H + 3) / 4;
     if (range_fits(in)) {
         // the allocation of this frame may have filled the range already
         cudaError_t e = range_ready ? cudaSuccess : launch_raycast_range(s, in, M_d, s.range_min, s.range_max, st);
-        // bit 1 of order_side: the header of side order_side & 1 is already
-        // clear (the previous raycast's finish kernel cleared it); it is
-        // dropped first, so that a launch error below leaves it unset
-        const int w = order_side & 1;
-        const bool pre_cleared = (order_side & 2) != 0;
-        order_side = w;
-        int32_t *hdr_w = s.tile_q_hdr + w * kTileHdrInts, *list_w = s.tile_q_list + (size_t)w * kTileClasses * kOrderMaxTiles;
-        const int32_t *hdr_r = s.tile_q_hdr + (1 - w) * kTileHdrInts;
-        const int32_t *list_r = s.tile_q_list + (size_t)(1 - w) * kTileClasses * kOrderMaxTiles;
-        if (e == cudaSuccess && !pre_cleared) e = launch_pdl(zero_words_kernel, dim3(1), dim3(32), 0, st, hdr_w, kTileHdrInts);
         if (e != cudaSuccess) return e;
-        static int g_dyn[2] = {0, 0};
+        static int g_dyn[2] = {0, 0}, sms = 1;
         const int mode = s.weight_mode ? 1 : 0;
         if (!g_dyn[mode]) {
-            int dev = 0, sms = 1, per = 1;
+            int dev = 0, per = 1;
             cudaGetDevice(&dev);
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                &per, mode ? (const void *)raycast_dynamic_kernel<1> : (const void *)raycast_dynamic_kernel<0>, 256, 0);
+                &per, mode ? (const void *)raycast_march_kernel<1> : (const void *)raycast_march_kernel<0>, 256, 0);
             g_dyn[mode] = sms * (per > 0 ? per : 1);
         }
-        const int n_tiles = tx * ty;
-        const int g = g_dyn[mode] < (n_tiles + 7) / 8 ? g_dyn[mode] : (n_tiles + 7) / 8;
-        const bool write_order = n_tiles <= kOrderMaxTiles;
-        const bool use_order = write_order && order_dims[0] == tx && order_dims[1] == ty;
-        const float tBm = tB_m;
-        if (mode == 0)
-            e = launch_pdl(raycast_dynamic_kernel<0>, dim3(g), dim3(256), 0, st, s, in, T_wc, vtx, nrm, max_iter, tBm,
-                           inv_sv, (const uint32_t *)s.range_min, (const uint32_t *)s.range_max, tx, n_tiles, hdr_w,
-                           list_w, hdr_r, list_r, use_order, write_order);
-        else
-            e = launch_pdl(raycast_dynamic_kernel<1>, dim3(g), dim3(256), 0, st, s, in, T_wc, vtx, nrm, max_iter, tBm,
-                           inv_sv, (const uint32_t *)s.range_min, (const uint32_t *)s.range_max, tx, n_tiles, hdr_w,
-                           list_w, hdr_r, list_r, use_order, write_order);
+        const int n_tiles = tx * ty, ctas = (n_tiles + 7) / 8;
+        const int g = g_dyn[mode] < ctas ? g_dyn[mode] : ctas;
+        // CTAs for the slow rays, three per SM (of four that fit beside each
+        // other; with one 640x480 takes 158 us instead of 129, 2 mm 798
+        // instead of 731); none for an image that could have more than the
+        // list holds.  room, the list's length up to which warps give rays up
+        // early: as many as these take at once, but at most 48 per SM: with
+        // all 192 the room takes 129 us instead of 136 and the 2 mm hall, a
+        // third of whose rays are slow, 731 instead of 679 (with none, that is
+        // after 48 iterations only, 140 and 681; 160x120 59 and 70).
+        const int slow_ctas = (long long)in.W * in.H > kSlowMax ? 0 : 3 * sms < ctas ? 3 * sms : ctas;
+        const uint32_t *rmin = s.range_min, *rmax = s.range_max;
+        const auto march = mode ? raycast_march_kernel<1> : raycast_march_kernel<0>;
+        const auto finish = mode ? raycast_finish_kernel<1> : raycast_finish_kernel<0>;
+        e = launch_pdl(march, dim3(g), dim3(256), 0, st, s, in, T_wc, vtx, max_iter, tB_m, inv_sv, rmin, rmax, tx,
+                       n_tiles, 64 * slow_ctas < 48 * sms ? 64 * slow_ctas : 48 * sms);
         if (e != cudaSuccess) return e;
-        // with write_order the next raycast writes side 1 - w, which this
-        // one only read: the finish kernel clears its header
-        int32_t *hdr_clear = write_order ? s.tile_q_hdr + (1 - w) * kTileHdrInts : nullptr;
-        if (mode == 0)
-            e = launch_pdl(raycast_finish_kernel<0>, grid, dim3(256), 0, st, s, in, T_wc, vtx, nrm, max_iter, tBm, inv_sv,
-                           hdr_clear);
-        else
-            e = launch_pdl(raycast_finish_kernel<1>, grid, dim3(256), 0, st, s, in, T_wc, vtx, nrm, max_iter, tBm, inv_sv,
-                           hdr_clear);
-        if (e != cudaSuccess) return e;
-        if (write_order) {
-            order_dims[0] = tx;
-            order_dims[1] = ty;
-            order_side = (1 - w) | 2;
-        }
-        return cudaSuccess;
-    } else {
-        if (s.weight_mode == 0)
-            raycast_kernel<0, false><<<grid, 256, 0, st>>>(s, in, T_wc, vtx, nrm, max_iter, tB_m, inv_sv, nullptr,
-                                                           nullptr, tx, ty);
-        else
-            raycast_kernel<1, false><<<grid, 256, 0, st>>>(s, in, T_wc, vtx, nrm, max_iter, tB_m, inv_sv, nullptr,
-                                                           nullptr, tx, ty);
+        return launch_pdl(finish, dim3(slow_ctas + ctas), dim3(256), 0, st, s, in, T_wc, vtx, nrm, max_iter, tB_m,
+                          inv_sv, rmin, rmax, tx, n_tiles, slow_ctas);
     }
+    const auto whole = s.weight_mode ? raycast_kernel<1> : raycast_kernel<0>;
+    whole<<<grid, 256, 0, st>>>(s, in, T_wc, vtx, nrm, max_iter, tB_m, inv_sv);
     return cudaGetLastError();
 }
 
