@@ -268,13 +268,15 @@ __global__ void __launch_bounds__(kIcpThreads) icp_step_kernel(
     };
     if (prefetch) camera_points();
     grid_dep_wait();
-    if (st && __ldcg(&st->done_level) == level) return;
-    if (!prefetch) camera_points();
     Mat34 T = T_arg;
     if (st) {
+        // the pose with the level's flag, not after it
+        const int done_level = __ldcg(&st->done_level);
 #pragma unroll
         for (int k = 0; k < 12; ++k) T.m[k] = __ldcg(&st->T[k]);
+        if (done_level == level) return;
     }
+    if (!prefetch) camera_points();
     const float t2 = fmul(dist_thresh, dist_thresh);
     float acc[32];
 #pragma unroll
