@@ -101,9 +101,18 @@ __global__ void __launch_bounds__(256) build_visible_kernel(SceneDev s, Mat34 M,
     const int n = min(__ldcg(&s.ctr->block_head), s.nv), head_before = __ldcg(&s.ctr->head_before);
     const float zfar = visible_zfar(s, frame_set(s));
     const int groups = gridDim.x * (blockDim.x >> 3);
+    // a group's next block is fetched (two dependent loads) beside the test of this one
+    int i = blockIdx.x * (blockDim.x >> 3) + (threadIdx.x >> 3);
+    int ptr = i < n ? __ldg(&s.block_free[i]) : 0;
+    short4 b = i < n ? __ldcg(&s.block_pos[ptr]) : make_short4(0, 0, 0, 0);
     for (int g0 = blockIdx.x * (blockDim.x >> 3); g0 < n; g0 += groups) {
-        const int i = g0 + (threadIdx.x >> 3);
-        visible_8<RANGE>(s, M, in, zfar, head_before, i < n, i, zc, tiles_x, tiles_y);
+        const int i_next = i + groups;
+        const int ptr_next = i_next < n ? __ldg(&s.block_free[i_next]) : 0;
+        const short4 b_next = i_next < n ? __ldcg(&s.block_pos[ptr_next]) : make_short4(0, 0, 0, 0);
+        visible_8<RANGE>(s, M, in, zfar, i >= head_before, ptr, b, zc, tiles_x, tiles_y);
+        i = i_next;
+        ptr = ptr_next;
+        b = b_next;
     }
     grid_dep_launch();
 }
