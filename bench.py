@@ -843,7 +843,7 @@ def run_tracking_section(itm, torch, dev, stream, scene, raw_dev, poses, ci, dep
         "steps_per_track": sum(TRACK_ITERS),
         "translation_error_mm_mean": 1000.0 * float(np.mean(err_t)),
         "rotation_error_deg_mean": float(np.mean(err_a)),
-        "reduce_full_res": {"kernel": "icp_partial_kernel + icp_solve_kernel", "bound": "hbm",
+        "reduce_full_res": {"kernel": "icp_step_kernel + icp_sum_kernel", "bound": "hbm",
                             "ms": red, "pixels_used_mean": float(np.mean(used)),
                             "algorithmic_bytes": alg, "achieved_gbs": alg / (red / 1000.0) / 1e9,
                             "peak": peak, "peak_kind": peak_kind, "frac": alg / (red / 1000.0) / 1e9 / peak},
@@ -1355,9 +1355,9 @@ def run_ours(args, world, rank, local):
         "cpu_baseline_threaded": cpu_mt,
         "clocks": clocks,
         "e2e": e2e,
-        # per frame: counter reset, enumerate (+ u16), commit (+ overflow), visible + range, integrate, raycast
-        # march, raycast finish (which clears the next raycast's tile-queue header)
-        "gpu_launches": 7 * args.steps,
+        # per frame: enumerate (+ u16), commit (+ overflow), visible + range, integrate, raycast march, raycast
+        # finish (+ slow rays)
+        "gpu_launches": 6 * args.steps,
         "batched": batched_rep,
         "learned": learned_rep,
         "tracking": tracking_rep,
