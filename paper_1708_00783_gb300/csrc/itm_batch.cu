@@ -11,7 +11,7 @@
 // virtual index is mapped back to its item by binary search, and the item's
 // work runs through the same bodies as the single-scene kernels (itm_ops.cuh),
 // so each scene gets bit-identical arithmetic.  Because no launch depends on
-// the work sizes, the eight launches are captured once into a CUDA graph and
+// the work sizes, the nine launches are captured once into a CUDA graph and
 // replayed for any item set up to the batch's capacity: per frame the host
 // only uploads the item table (pinned ring buffer, one async copy) and
 // launches the graph.

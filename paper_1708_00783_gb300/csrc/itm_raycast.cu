@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(256, 4) raycast_finish_kernel(SceneDev s, Intr
         c->entered = begun;
     }
     const int n_slow = cta < 0 ? min(__ldcg(&c->set[(begun - 1u) & 1u].n_slow), kSlowMax) : 0;
-    const int rounds = min((n_slow - 1) / (64 * slow_ctas) + 1, 4);
+    const int rounds = n_slow > 0 ? min((n_slow - 1) / (64 * slow_ctas) + 1, 4) : 1;
     for (int g = cta < 0 ? (int)blockIdx.x + slow_ctas * warp : cta * 8 + warp;
          cta < 0 ? g * 8 * rounds < n_slow : g < tiles; g += cta < 0 ? 8 * slow_ctas : tiles) {
         const EndedRay e = cta < 0 ? raycast_slow_rays<MODE>(s, in, T, vtx, max_iter, tB_m, inv_sv, rmin, rmax, tiles_x,
