@@ -519,6 +519,9 @@ struct itm_scene {
     // allocation (made by itm_scene_create)
     cudaStream_t aux;
     cudaEvent_t ev_fork, ev_join;
+    // a raycast's march was launched and its finish could not be: the counts
+    // of rays (ray_ctr) are those of a raycast under way (recover)
+    bool rays_behind;
 };
 
 // An NVTX range named after a C-ABI call for the duration of the call, so
@@ -548,8 +551,9 @@ cudaError_t launch_allocate(const SceneDev &s, const float *depth, const Intr &i
 // these intrinsics, and no block changed since, so its interior flags hold
 cudaError_t launch_integrate(const SceneDev &s, const float *depth, const float *wpx, const Intr &in,
                              const Mat34 &M_d, bool interior_ok, cudaStream_t st);
+// half: the march was launched and the finish was not
 cudaError_t launch_raycast(const SceneDev &s, const Intr &in, const Mat34 &T_wc, const Mat34 &M_d, float4 *vtx,
-                           float4 *nrm, bool range_ready, cudaStream_t st);
+                           float4 *nrm, bool range_ready, cudaStream_t st, bool &half);
 cudaError_t launch_raycast_range(const SceneDev &s, const Intr &in, const Mat34 &M_d, uint32_t *rmin, uint32_t *rmax,
                                  cudaStream_t st);
 bool range_fits(const Intr &in);

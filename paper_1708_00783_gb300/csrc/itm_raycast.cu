@@ -176,8 +176,9 @@ cudaError_t launch_raycast_range(const SceneDev &s, const Intr &in, const Mat34 
 }
 
 cudaError_t launch_raycast(const SceneDev &s, const Intr &in, const Mat34 &T_wc, const Mat34 &M_d, float4 *vtx,
-                           float4 *nrm, bool range_ready, cudaStream_t st)
+                           float4 *nrm, bool range_ready, cudaStream_t st, bool &half)
 {
+    half = false;
     // host-side constants with the same float operations as the oracle
     volatile float span = s.z_max - s.z_min;
     volatile float four_span = 4.0f * span;
@@ -219,8 +220,10 @@ cudaError_t launch_raycast(const SceneDev &s, const Intr &in, const Mat34 &T_wc,
         e = launch_pdl(march, dim3(g), dim3(256), 0, st, s, in, T_wc, vtx, max_iter, tB_m, inv_sv, rmin, rmax, tx,
                        n_tiles, 64 * slow_ctas < 48 * sms ? 64 * slow_ctas : 48 * sms);
         if (e != cudaSuccess) return e;
-        return launch_pdl(finish, dim3(slow_ctas + ctas), dim3(256), 0, st, s, in, T_wc, vtx, nrm, max_iter, tB_m,
-                          inv_sv, rmin, rmax, tx, n_tiles, slow_ctas);
+        e = launch_pdl(finish, dim3(slow_ctas + ctas), dim3(256), 0, st, s, in, T_wc, vtx, nrm, max_iter, tB_m,
+                       inv_sv, rmin, rmax, tx, n_tiles, slow_ctas);
+        half = e != cudaSuccess;
+        return e;
     }
     const auto whole = s.weight_mode ? raycast_kernel<1> : raycast_kernel<0>;
     whole<<<grid, 256, 0, st>>>(s, in, T_wc, vtx, nrm, max_iter, tB_m, inv_sv);

@@ -88,6 +88,19 @@ static int valid_params(const itm_scene_params *p)
     return 1;
 }
 
+// Puts right what a call that failed between two of its launches left behind,
+// before the next call builds on it.  While st is being captured it stays
+// noted, as the work put into the capture has not run.
+static cudaError_t recover(itm_scene *sc, cudaStream_t st)
+{
+    if (!sc->rays_behind) return cudaSuccess;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(st, &cap);
+    if (e == cudaSuccess) e = cudaMemsetAsync(sc->d.ray_ctr, 0, sizeof(RayCounters), st);
+    if (e == cudaSuccess && cap == cudaStreamCaptureStatusNone) sc->rays_behind = false;
+    return e;
+}
+
 static void free_dev(SceneDev &d)
 {
     void *ptrs[] = {d.entries, d.req, d.req_list, d.overflow, d.visible, d.block_pos, d.sdf,
@@ -314,8 +327,14 @@ int itm_raycast(itm_scene *sc, const itm_intrinsics *intr, const float T_wc[16],
     sc->last_stream = st;
     const bool ready = sc->range_epoch == sc->alloc_epoch && memcmp(sc->range_pose, T_wc, sizeof(sc->range_pose)) == 0 &&
                        memcmp(&sc->range_intr, intr, sizeof(itm_intrinsics)) == 0;
-    const int r = check_cuda(launch_raycast(sc->d, to_intr(intr), T, M, reinterpret_cast<float4 *>(vertex_dev),
-                                            reinterpret_cast<float4 *>(normal_dev), ready, st));
+    if (!ready && range_fits(to_intr(intr))) sc->range_epoch = -1;  // the range tiles are written for this pose
+    bool half = false;
+    cudaError_t e = recover(sc, st);
+    if (e == cudaSuccess)
+        e = launch_raycast(sc->d, to_intr(intr), T, M, reinterpret_cast<float4 *>(vertex_dev),
+                           reinterpret_cast<float4 *>(normal_dev), ready, st, half);
+    if (half) sc->rays_behind = true;
+    const int r = check_cuda(e);
     if (r == ITM_OK && range_fits(to_intr(intr))) {
         sc->range_epoch = sc->alloc_epoch;
         memcpy(sc->range_pose, T_wc, sizeof(sc->range_pose));
