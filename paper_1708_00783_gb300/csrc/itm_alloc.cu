@@ -140,8 +140,9 @@ int persistent_grid(int threads, const void *kernel)
 }  // namespace
 
 cudaError_t launch_allocate(const SceneDev &s, const float *depth, const Intr &in, const Mat34 &T_wc,
-                            const Mat34 &M_d, bool with_range, cudaStream_t st, const uint16_t *raw)
+                            const Mat34 &M_d, bool with_range, cudaStream_t st, const uint16_t *raw, bool &half)
 {
+    half = false;
     const float inv_b = (float)(1.0 / (8.0 * (double)s.voxel_size));
     dim3 grid((in.W + 31) / 32, (in.H + 7) / 8);
     const int n_range_tiles = with_range ? ((in.W + 7) / 8) * ((in.H + 3) / 4) : 0;
@@ -163,6 +164,7 @@ cudaError_t launch_allocate(const SceneDev &s, const float *depth, const Intr &i
     } else {
         e = launch_pdl(build_visible_kernel<false>, dim3(g_visible), dim3(256), 0, st, s, M_d, in, 0.0f, 1, 1);
     }
+    half = e != cudaSuccess;
     return e;
 }
 

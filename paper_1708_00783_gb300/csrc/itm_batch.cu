@@ -529,8 +529,10 @@ int itm_batch_run(itm_batch *b, const itm_batch_item *items, int n, itm_stream s
     h->cta_total = cta_total;
     h->scatter_p = scatter_multiplier(cta_total);
     h->pad = 0;
-    cudaError_t e = cudaMemcpyAsync(b->d_head, h, sizeof(BatchHead) + sizeof(ItemDev) * (size_t)n,
-                                    cudaMemcpyHostToDevice, st);
+    cudaError_t e = cudaSuccess;
+    for (int i = 0; i < n && e == cudaSuccess; ++i) e = recover(items[i].scene, st);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(b->d_head, h, sizeof(BatchHead) + sizeof(ItemDev) * (size_t)n, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaEventRecord(b->ev[slot], st);
     if (e != cudaSuccess) return ITM_ERR_CUDA;
     if (b->use_graph && st != nullptr) {

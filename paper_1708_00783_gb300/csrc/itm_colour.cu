@@ -248,6 +248,8 @@ int itm_colour_at(itm_scene *sc, const float *points_dev, int64_t n, uint8_t *rg
     if (n == 0) return ITM_OK;
     cudaStream_t st = (cudaStream_t)stream;
     sc->last_stream = st;
+    const cudaError_t e = recover(sc, st);
+    if (e != cudaSuccess) return check_cuda(e);
     const float inv_sv = (float)(1.0 / (double)sc->d.voxel_size);
     const int g = (int)std::min<int64_t>((n + 255) / 256, (int64_t)grid_for(8));
     colour_at_kernel<<<g, 256, 0, st>>>(sc->d, reinterpret_cast<const float4 *>(points_dev), n, inv_sv, sc->d.rgbw,

@@ -106,6 +106,13 @@ cudaError_t launch_brick_fill(const SceneDev &s, int n, cudaStream_t st)
     return cudaGetLastError();
 }
 
+cudaError_t launch_brick_refill(const SceneDev &s, cudaStream_t st)
+{
+    brick_reset_kernel<<<stream_grid(), 256, 0, st>>>(s);
+    const cudaError_t e = cudaGetLastError();
+    return e != cudaSuccess ? e : launch_brick_fill(s, s.nv, st);
+}
+
 cudaError_t launch_depth_u16(const uint16_t *raw, float *out, int64_t n, cudaStream_t st)
 {
     if (n <= 0) return cudaSuccess;

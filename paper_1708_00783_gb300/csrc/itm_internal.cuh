@@ -216,8 +216,10 @@ __device__ __forceinline__ int lookup_cg(const SceneDev &s, int bx, int by, int 
 
 // ----------------------------------------------------------- brick table
 // The blocks in device memory by their coordinates, for the kernels that look
-// blocks up without changing them (the raycasts, the mesh, the colour of
-// points): beside the hash table, which stays what decides.  A brick is 8 x 8
+// blocks up without changing them: the raycasts, the mesh, the colour of
+// points, and the enumeration, which requests a block when it is not found
+// here, so that every block of the hash table has to be here as well (or its
+// brick marked) before the next allocation begins.  A brick is 8 x 8
 // x 8 blocks, brick (X, Y, Z) = (bx, by, bz) >> 3; its place in the table is a
 // hash of its coordinates.  A place has room for one brick, the first that
 // came (brick_owner), and holds 9 x 9 x 9 block indices: the brick's blocks
@@ -236,9 +238,11 @@ __device__ __forceinline__ int lookup_cg(const SceneDev &s, int bx, int by, int 
 // the room; cells with a tag of their own instead of the place's owner took a
 // fifth more instructions.)
 //
-// Blocks enter in the pass of the allocation that hands them out (and after an
-// import), and leave in the swap-out; the kernels that change the table and
-// those that read it never run at the same time.
+// Blocks enter in the last pass of the allocation that hands them out (and
+// after an import), and leave in the swap-out; the kernels that change the
+// table and those that read it never run at the same time.  When that pass
+// cannot be launched, the scene notes it and the next call enters all blocks
+// anew (recover).
 constexpr int kBrickSide = 9;      // blocks along a brick's edge with the one further
 constexpr int kBrickCells = 736;   // 9^3 cells, rounded up to whole 32-byte sectors
 constexpr int kBrickMin = 4096;    // smallest number of places (12 MB)
@@ -522,6 +526,9 @@ struct itm_scene {
     // a raycast's march was launched and its finish could not be: the counts
     // of rays (ray_ctr) are those of a raycast under way (recover)
     bool rays_behind;
+    // the same of an allocation's commit and its visible-list pass: blocks that
+    // the hash table has are not in the brick table
+    bool bricks_behind;
 };
 
 // An NVTX range named after a C-ABI call for the duration of the call, so
@@ -541,12 +548,16 @@ Intr to_intr(const itm_intrinsics *in);
 // the visible list's interior flags hold for an integration with this pose
 // and these intrinsics (launch_integrate's interior_ok)
 bool interior_flags_hold(const itm_scene *sc, const float T_wc[16], const itm_intrinsics *intr);
+// Puts right what a call that failed between two of its launches left behind;
+// every call that reads or changes the brick table or the ray counts begins with it.
+cudaError_t recover(itm_scene *sc, cudaStream_t st);
 }  // namespace itm
 
 // Launchers implemented in the kernel translation units.
 namespace itm {
+// half: the commit was launched and the visible-list pass was not
 cudaError_t launch_allocate(const SceneDev &s, const float *depth, const Intr &in, const Mat34 &T_wc,
-                            const Mat34 &M_d, bool with_range, cudaStream_t st, const uint16_t *raw = nullptr);
+                            const Mat34 &M_d, bool with_range, cudaStream_t st, const uint16_t *raw, bool &half);
 // interior_ok: the visible list was built by an allocation with this pose and
 // these intrinsics, and no block changed since, so its interior flags hold
 cudaError_t launch_integrate(const SceneDev &s, const float *depth, const float *wpx, const Intr &in,
@@ -577,4 +588,6 @@ cudaError_t launch_raycast_merge(const float4 *vtx, const float4 *nrm, int parts
 cudaError_t launch_reset(const SceneDev &s, cudaStream_t st);
 // enters blocks 0 .. n-1 (block_pos) in the brick table
 cudaError_t launch_brick_fill(const SceneDev &s, int n, cudaStream_t st);
+// empties the brick table and enters every block in use
+cudaError_t launch_brick_refill(const SceneDev &s, cudaStream_t st);
 }  // namespace itm

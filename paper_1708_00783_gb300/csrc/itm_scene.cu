@@ -88,16 +88,16 @@ static int valid_params(const itm_scene_params *p)
     return 1;
 }
 
-// Puts right what a call that failed between two of its launches left behind,
-// before the next call builds on it.  While st is being captured it stays
-// noted, as the work put into the capture has not run.
-static cudaError_t recover(itm_scene *sc, cudaStream_t st)
+// While st is being captured the state stays noted, as the work put into the
+// capture has not run (clearing and filling again once more does no harm).
+cudaError_t recover(itm_scene *sc, cudaStream_t st)
 {
-    if (!sc->rays_behind) return cudaSuccess;
+    if (!sc->rays_behind && !sc->bricks_behind) return cudaSuccess;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     cudaError_t e = cudaStreamIsCapturing(st, &cap);
-    if (e == cudaSuccess) e = cudaMemsetAsync(sc->d.ray_ctr, 0, sizeof(RayCounters), st);
-    if (e == cudaSuccess && cap == cudaStreamCaptureStatusNone) sc->rays_behind = false;
+    if (e == cudaSuccess && sc->rays_behind) e = cudaMemsetAsync(sc->d.ray_ctr, 0, sizeof(RayCounters), st);
+    if (e == cudaSuccess && sc->bricks_behind) e = launch_brick_refill(sc->d, st);
+    if (e == cudaSuccess && cap == cudaStreamCaptureStatusNone) sc->rays_behind = sc->bricks_behind = false;
     return e;
 }
 
@@ -235,7 +235,11 @@ int itm_scene_reset(itm_scene *sc, itm_stream stream)
     sc->vis_ok = false;
     cudaStream_t st = (cudaStream_t)stream;
     sc->last_stream = st;
-    cudaError_t e = launch_reset(sc->d, st);
+    cudaError_t e = recover(sc, st);
+    if (e == cudaSuccess) {
+        e = launch_reset(sc->d, st);
+        sc->bricks_behind |= e != cudaSuccess;
+    }
     if (e == cudaSuccess) e = swap_reset(sc, st);
     if (e == cudaSuccess && sc->d.rgbw)
         e = cudaMemsetAsync(sc->d.rgbw, 0, sizeof(uint32_t) * (size_t)(sc->d.nv > 0 ? sc->d.nv : 1) * kBlockVoxels, st);
@@ -256,7 +260,11 @@ static int allocate_impl(itm_scene *sc, const float *depth_dev, const uint16_t *
     sc->alloc_epoch++;
     sc->vis_ok = false;
     if (sc->d.swap_state) sc->d.swap_frame++;  // Sec. 5: the blocks this allocation meets are stamped with it
-    const int r = check_cuda(launch_allocate(sc->d, depth_dev, in, T, M, with_range, st, raw_dev));
+    bool half = false;
+    cudaError_t e = recover(sc, st);
+    if (e == cudaSuccess) e = launch_allocate(sc->d, depth_dev, in, T, M, with_range, st, raw_dev, half);
+    if (half) sc->bricks_behind = true;
+    const int r = check_cuda(e);
     if (r == ITM_OK) {
         // the visible list's interior flags hold for this pose and these intrinsics
         sc->vis_ok = true;
@@ -414,7 +422,11 @@ int itm_raycast_combined(itm_scene *const *scenes, const float *submap_from_worl
     pose_rows(T_wc, T);
     // the combined raycast writes its search ranges into the submaps' range
     // scratch: their next itm_raycast recomputes its own
-    for (int i = 0; i < n; ++i) scenes[i]->range_epoch = -1;
+    for (int i = 0; i < n; ++i) {
+        scenes[i]->range_epoch = -1;
+        const cudaError_t e = recover(scenes[i], (cudaStream_t)stream);
+        if (e != cudaSuccess) return check_cuda(e);
+    }
     return check_cuda(launch_raycast_combined(subs, P, n, to_intr(intr), T, reinterpret_cast<float4 *>(vertex_dev),
                                               reinterpret_cast<float4 *>(normal_dev), (cudaStream_t)stream));
 }
@@ -546,7 +558,8 @@ int itm_mesh(itm_scene *sc, float *triangles_dev, int64_t capacity, int64_t *n_o
     cudaStream_t st = (cudaStream_t)stream;
     sc->last_stream = st;
     unsigned long long *counter = &sc->d.ctr->mesh_tris;
-    cudaError_t e = launch_mesh(sc->d, triangles_dev, (long long)capacity, counter, st);
+    cudaError_t e = recover(sc, st);
+    if (e == cudaSuccess) e = launch_mesh(sc->d, triangles_dev, (long long)capacity, counter, st);
     unsigned long long cnt = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&cnt, counter, sizeof(cnt), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -781,6 +794,7 @@ int itm_scene_import(itm_scene *sc, const int16_t *coords_host, const float *sdf
     sc->alloc_epoch++;
     sc->vis_ok = false;
     cudaError_t e = cudaStreamSynchronize(sc->last_stream);
+    sc->bricks_behind = true;  // until the new volume's blocks are entered
     if (e == cudaSuccess) e = launch_reset(d, 0);
     if (e == cudaSuccess) e = swap_reset(sc, 0);
     if (e == cudaSuccess && d.rgbw)
@@ -804,7 +818,10 @@ int itm_scene_import(itm_scene *sc, const int16_t *coords_host, const float *sdf
         e = cudaMemcpy(d.ctr, &c, sizeof(c), cudaMemcpyHostToDevice);
     }
     if (e == cudaSuccess) e = launch_brick_fill(d, n, 0);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(0);
+    if (e == cudaSuccess) {
+        sc->bricks_behind = false;
+        e = cudaStreamSynchronize(0);
+    }
     sc->last_stream = 0;
     return check_cuda(e);
 }

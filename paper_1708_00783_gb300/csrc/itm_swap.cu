@@ -553,7 +553,8 @@ int itm_swap_out(itm_scene *sc, itm_stream stream)
     cudaStream_t st = (cudaStream_t)stream;
     sc->last_stream = st;
     const SwapDev w = swap_dev(sc);
-    cudaError_t e = launch_select<true>(sc->d, w, st);
+    cudaError_t e = recover(sc, st);
+    if (e == cudaSuccess) e = launch_select<true>(sc->d, w, st);
     if (e != cudaSuccess) return check_cuda(e);
     if (sc->d.weight_mode == 0)
         swap_out_kernel<0><<<move_grid(w.k), kMoveThreads, 0, st>>>(sc->d, w);

@@ -106,3 +106,132 @@ for n, before, k in ((1, 9, 9), (2, 9, 9), (2, 9, 2), (3, 9, 2), (2, 2, 2), (2, 
         g.raycast(ci, pose(again), *got)
         assert same(got, want[again]), (n, before, k, again)
 """)
+
+
+# what follows an allocation of which the commit ran and the visible-list pass did not
+AFTER = {
+    "allocate": r"""
+for s in (g, o):
+    s.process(depth(9), ci, pose(9), *maps())
+""",
+    "raycast": r"""
+m = [maps(), maps()]
+for s, x in ((g, m[0]), (o, m[1])):
+    s.raycast(ci, pose(9), *x)
+assert same(*m)
+""",
+    "mesh": r"""
+a, b = gpu_mesh(itm, g), gpu_mesh(itm, o)
+assert len(a) > 0 and np.array_equal(canonical(a), canonical(b))
+""",
+    "combined": r"""
+m = [maps(), maps()]
+eye = np.eye(4, dtype=np.float32)[None]
+for s, x in ((g, m[0]), (o, m[1])):
+    itm.itm_raycast_combined([s.handle], eye, ci, pose(9), *x)
+assert same(*m)
+""",
+    "batch": r"""
+b = itm.itm_batch_create(1)
+m = [maps(), maps()]
+for s, x in ((g, m[0]), (o, m[1])):
+    itm.itm_batch_run(b, [(s.handle, depth(9), ci, pose(9), x[0], x[1])])
+assert same(*m)
+""",
+    "swap_out": r"""
+for s in (g, o):
+    s.swap_out()
+    for k in (9, 0, 5, 9):
+        s.allocate(depth(k), ci, pose(k))
+        s.swap_in()
+        s.integrate(depth(k), ci, pose(k))
+        s.swap_out()
+assert g.swap_counters()["moved_out"] == o.swap_counters()["moved_out"] > 0
+""",
+    "reset": r"""
+for s in (g, o):
+    s.reset()
+    s.process(depth(5), ci, pose(5), *maps())
+""",
+    "import": r"""
+v = g.export()
+for s in (g, o):
+    s.import_blocks(*v)
+""",
+}
+
+
+@pytest.mark.parametrize("then", sorted(AFTER))
+def test_allocation_without_its_visible_list(package, then):
+    """The blocks of the refused frame are found by whatever comes next, and no key is entered twice."""
+    run(package, r"""
+g, o = itm.Scene(**w.params), itm.Scene(**w.params)
+if %r == "swap_out":
+    for s in (g, o):
+        s.swap_enable(4096, 0)
+for s in (g, o):
+    for k in (0, 1):
+        s.process(depth(k), ci, pose(k), *maps())
+before = g.stats()["allocated_blocks"]
+refused(3, lambda: g.allocate(depth(9), ci, pose(9)))
+o.allocate(depth(9), ci, pose(9))
+assert g.stats()["allocated_blocks"] > before + 100
+""" % then + AFTER[then] + r"""
+assert g.status() == o.status() == 0
+assert same_volume(g, o)
+for k in (9, 5, 0):
+    for s in (g, o):
+        s.allocate(depth(k), ci, pose(k))
+        if %r == "swap_out":
+            s.swap_in()
+        s.integrate(depth(k), ci, pose(k))
+    m = [maps(), maps()]
+    g.raycast(ci, pose(k), *m[0])
+    o.raycast(ci, pose(k), *m[1])
+    assert same(*m), k
+assert same_volume(g, o) and g.status() == o.status() == 0
+""" % then)
+
+
+@pytest.mark.parametrize("n", [1, 2])
+def test_allocation_refused_before(package, n):
+    """The enumeration or the commit refused: the frame can be repeated."""
+    run(package, r"""
+g, o = itm.Scene(**w.params), itm.Scene(**w.params)
+for s in (g, o):
+    s.process(depth(0), ci, pose(0), *maps())
+refused(%d, lambda: g.allocate(depth(9), ci, pose(9)))
+for k in (9, 5):
+    m = [maps(), maps()]
+    g.process(depth(k), ci, pose(k), *m[0])
+    o.process(depth(k), ci, pose(k), *m[1])
+    assert same(*m), k
+    assert g.stats()["allocated_blocks"] == o.stats()["allocated_blocks"]
+assert same_volume(g, o) and g.status() == o.status() == 0
+""" % n)
+
+
+def test_import_and_reset(package):
+    """Every launch of an import and of a reset refused in turn, then done again."""
+    run(package, r"""
+g, o = itm.Scene(**w.params), itm.Scene(**w.params)
+for s in (g, o):
+    s.process(depth(0), ci, pose(0), *maps())
+v = o.export()
+for n in (1, 2, 3, 4):
+    refused(n, lambda: g.import_blocks(*v))
+    for _ in range(2):  # what the failed one left is not the volume: import again
+        g.import_blocks(*v)
+    m = [maps(), maps()]
+    g.raycast(ci, pose(0), *m[0])
+    o.raycast(ci, pose(0), *m[1])
+    assert same(*m) and same_volume(g, o), n
+for n in (1, 2, 3):
+    refused(n, g.reset)
+    g.reset()
+    m = [maps(), maps()]
+    g.process(depth(0), ci, pose(0), *m[0])
+    o.reset()
+    o.process(depth(0), ci, pose(0), *m[1])
+    assert same(*m) and same_volume(g, o), n
+""")
