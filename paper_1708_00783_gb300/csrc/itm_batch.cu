@@ -138,6 +138,9 @@ __global__ void __launch_bounds__(256) batch_commit_kernel(const ItemDev *__rest
         const int k = find_item(prefix, n, i);
         commit_request(items[k].s, i - prefix[k]);
     }
+    // here and not in a later stage: a frame whose requests are entered is over for the counts
+    if (blockIdx.x == 0)
+        for (int k = threadIdx.x; k < n; k += blockDim.x) frame_end(items[k].s);
 }
 
 __global__ void __launch_bounds__(kOvfThreads) batch_overflow_kernel(const ItemDev *__restrict__ items,
@@ -147,7 +150,6 @@ __global__ void __launch_bounds__(kOvfThreads) batch_overflow_kernel(const ItemD
     if ((int)blockIdx.x >= head->n) return;
     const SceneDev &s = items[blockIdx.x].s;
     overflow_scene(s, __ldcg(&frame_set(s)->n_overflow), remaining);
-    if (threadIdx.x == 0) frame_end(s);
 }
 
 __global__ void __launch_bounds__(256) batch_visible_kernel(const ItemDev *__restrict__ items, const BatchHead *head)
@@ -351,19 +353,30 @@ static void drop_graph(itm_batch *b)
     }
 }
 
+// The first launch that is refused ends the batch: a stage that ran without
+// the one before it would work on the counts of an earlier frame.
 static cudaError_t launch_stages(itm_batch *b, cudaStream_t st)
 {
     const ItemDev *it = b->d_items;
     const BatchHead *h = b->d_head;
+    cudaError_t e;
     batch_begin_kernel<<<b->max_items, 256, 0, st>>>(it, h);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     batch_enumerate_kernel<<<b->grid[ST_ENUM], 256, 0, st>>>(it, h, b->knob[K_ENUM_SCATTER] != 0);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     batch_commit_kernel<<<b->grid[ST_COMMIT], 256, 0, st>>>(it, h);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     batch_overflow_kernel<<<b->max_items, kOvfThreads, 0, st>>>(it, h);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     batch_visible_kernel<<<b->grid[ST_VISIBLE], 256, 0, st>>>(it, h);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     batch_integrate_kernel<<<b->grid[ST_INTEGRATE], stage_threads(b, ST_INTEGRATE), 0, st>>>(it, h,
                                                                                         make_float2(-0.0f, -0.0f));
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     batch_range_kernel<<<b->grid[ST_RANGE], 256, 0, st>>>(it, h);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     batch_raycast_kernel<<<b->grid[ST_RAYCAST], 256, 0, st>>>(it, h, b->knob[K_RAY_SCATTER] != 0);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     batch_finish_kernel<<<b->grid[ST_RAYCAST], 256, 0, st>>>(it, h, b->knob[K_RAY_SCATTER] != 0);
     return cudaGetLastError();
 }
@@ -555,6 +568,7 @@ int itm_batch_run(itm_batch *b, const itm_batch_item *items, int n, itm_stream s
         items[i].scene->last_stream = st;
         items[i].scene->alloc_epoch++;  // the batch rewrote the scene's range tiles
         items[i].scene->vis_ok = false;  // and its visible list
+        if (e != cudaSuccess) items[i].scene->bricks_behind = true;  // the visible-list stage may not have run
     }
     return check_cuda(e);
 }

@@ -235,3 +235,35 @@ for n in (1, 2, 3):
     o.process(depth(0), ci, pose(0), *m[1])
     assert same(*m) and same_volume(g, o), n
 """)
+
+
+@pytest.mark.parametrize("n", range(1, 10))
+def test_batch(package, n):
+    """Each launch of a batch without a captured graph refused in turn, then the frame once more."""
+    run(package, r"""
+scenes = []
+for p in (w.params, dict(w.params, num_buckets=1 << 8, num_excess=1 << 13)):
+    scenes.append((itm.Scene(**p), itm.Scene(**p)))
+b = itm.itm_batch_create(4)
+itm.itm_batch_set_graph(b, 0)
+
+def frame(side, k):
+    m = [maps() for _ in scenes]
+    items = [(s[side].handle, depth(k), ci, pose(k), v, n) for s, (v, n) in zip(scenes, m)]
+    itm.itm_batch_run(b, items)
+    return m
+
+for k in (0, 1):
+    frame(0, k), frame(1, k)
+refused(%d, lambda: frame(0, 9))
+if %d <= 6:  # stages: begin, enumerate, commit, overflow, visible, integrate, range, march, finish
+    frame(0, 9)
+frame(1, 9)
+for k in (5, 0):
+    for x, y in zip(frame(0, k), frame(1, k)):
+        assert same(x, y), k
+for g, o in scenes:
+    assert g.status() == o.status() == 0
+    assert g.stats()["allocated_blocks"] == len(g.export(False)[0])
+    assert same_volume(g, o)
+""" % (n, n))
