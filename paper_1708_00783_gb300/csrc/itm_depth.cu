@@ -84,7 +84,7 @@ __global__ void __launch_bounds__(256) brick_reset_kernel(SceneDev s)
         for (int i = lane; i < kBrickCells / 4; i += 32) cell[i] = make_int4(-1, -1, -1, -1);
         if (lane == 0) {
             s.brick_owner[p] = 0ull;
-            s.brick_count[p] = 0;
+            s.brick_count[p] = 0ull;
         }
     }
 }

@@ -108,7 +108,7 @@ struct SceneDev {
     int32_t *excess_free;
     Counters *ctr;
     unsigned long long *brick_owner;  // the brick of each place (brick_key), 0: none yet
-    int32_t *brick_count;             // cells of the place that hold a block
+    unsigned long long *brick_count;  // cells of the place that hold a block, kBrickOther for each block not entered
     int32_t *brick_cell;              // kBrickCells block indices per place, -1: none
     uint32_t brick_mask;              // places - 1
     uint32_t *range_min;  // per 8x4 tile: nearest / farthest depth (float bits) of covering blocks
@@ -226,7 +226,10 @@ __device__ __forceinline__ int lookup_cg(const SceneDev &s, int bx, int by, int 
 // and the blocks one further along each axis, so that the up to eight blocks
 // that a 2x2x2 voxel stencil reaches are cells of one brick at fixed offsets.
 // Blocks of a brick whose place is taken are not entered; the place is marked
-// (kBrickShared) and lookups in that brick go to the hash table.
+// (kBrickShared) and lookups in that brick go to the hash table.  They are
+// counted, so that the mark goes with the last of them, and a place that no
+// block counts on is free again: a camera that travels, with swapping, leaves
+// no places behind that are taken or marked for bricks that have left.
 //
 // Why: through the hash table each of those eight blocks was a key, a hash
 // and a scattered 16-byte load of its own, one after the other wherever any
@@ -246,10 +249,10 @@ __device__ __forceinline__ int lookup_cg(const SceneDev &s, int bx, int by, int 
 constexpr int kBrickSide = 9;      // blocks along a brick's edge with the one further
 constexpr int kBrickCells = 736;   // 9^3 cells, rounded up to whole 32-byte sectors
 constexpr int kBrickMin = 4096;    // smallest number of places (12 MB)
-constexpr unsigned long long kBrickValid = 1ull << 48, kBrickShared = 1ull << 63;
+constexpr unsigned long long kBrickValid = 1ull << 48, kBrickShared = 1ull << 63, kBrickOther = 1ull << 32;
 
 // places for nv blocks: one for every 16 blocks (a surface fills a brick with
-// about a hundred, and the bricks before it by their ninth cells), 184 bytes
+// about a hundred, and the bricks before it by their ninth cells), 185 bytes
 // per block beside its 2560 bytes of voxels.  Bricks that find their place
 // taken cost the walks the table is there to save: with one place for 32
 // blocks, 512 at least, a camera turning round in a room of 350 bricks took
@@ -384,26 +387,27 @@ __device__ __forceinline__ void brick_put(const SceneDev &s, int bx, int by, int
     const uint32_t place = brick_place(X, Y, Z, s.brick_mask);
     const unsigned long long key = brick_key(X, Y, Z);
     const unsigned long long old = atomicCAS(&s.brick_owner[place], 0ull, key);
-    if (old == 0ull || (old & ~kBrickShared) == key) {
-        s.brick_cell[(size_t)place * kBrickCells + local] = ptr;
-        atomicAdd(&s.brick_count[place], 1);
-    } else {
-        atomicOr(&s.brick_owner[place], kBrickShared);
-    }
+    const bool own = old == 0ull || (old & ~kBrickShared) == key;
+    if (own) s.brick_cell[(size_t)place * kBrickCells + local] = ptr;
+    else atomicOr(&s.brick_owner[place], kBrickShared);
+    atomicAdd(&s.brick_count[place], own ? 1ull : kBrickOther);
 }
 
-// The block at (bx, by, bz) leaves: the share of thread c (0..7).  A place
-// whose last block leaves is free again; a shared one never is (blocks of
-// other bricks may only be in the hash table).
+// The block at (bx, by, bz) leaves: the share of thread c (0..7).  While any
+// block counts on the place its owner stays, so this finds the owner that
+// brick_put found.  The one that takes the last count frees the place; the mark
+// may be taken off before or after that (a free place's word stays 0).
 __device__ __forceinline__ void brick_take(const SceneDev &s, int bx, int by, int bz, int c)
 {
     int X, Y, Z, local;
     if (!brick_share(bx, by, bz, c, X, Y, Z, local)) return;
     const uint32_t place = brick_place(X, Y, Z, s.brick_mask);
-    const unsigned long long own = __ldcg(&s.brick_owner[place]);
-    if ((own & ~kBrickShared) != brick_key(X, Y, Z)) return;
-    s.brick_cell[(size_t)place * kBrickCells + local] = -1;
-    if (atomicSub(&s.brick_count[place], 1) == 1 && !(own & kBrickShared)) s.brick_owner[place] = 0ull;
+    const bool own = (__ldcg(&s.brick_owner[place]) & ~kBrickShared) == brick_key(X, Y, Z);
+    if (own) s.brick_cell[(size_t)place * kBrickCells + local] = -1;
+    const unsigned long long one = own ? 1ull : kBrickOther;
+    const unsigned long long left = atomicAdd(&s.brick_count[place], 0ull - one) - one;
+    if (left == 0ull) s.brick_owner[place] = 0ull;
+    else if (left < kBrickOther && !own) atomicAnd(&s.brick_owner[place], ~kBrickShared);
 }
 
 // ------------------------------------------------------ slab partition

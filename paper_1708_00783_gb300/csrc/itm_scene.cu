@@ -181,7 +181,7 @@ int itm_scene_create(const itm_scene_params *params, itm_scene **out)
     const size_t places = (size_t)brick_places(d.nv);
     d.brick_mask = (uint32_t)(places - 1);
     ITM_ALLOC(d.brick_owner, sizeof(unsigned long long) * places);
-    ITM_ALLOC(d.brick_count, sizeof(int32_t) * places);
+    ITM_ALLOC(d.brick_count, sizeof(unsigned long long) * places);
     ITM_ALLOC(d.brick_cell, sizeof(int32_t) * kBrickCells * places);
     ITM_ALLOC(d.range_min, sizeof(uint32_t) * (size_t)kRangeMaxTiles);
     ITM_ALLOC(d.range_max, sizeof(uint32_t) * (size_t)kRangeMaxTiles);
@@ -195,7 +195,7 @@ int itm_scene_create(const itm_scene_params *params, itm_scene **out)
     }
     if (e == cudaSuccess) e = cudaMemsetAsync(d.ray_ctr, 0, sizeof(RayCounters), 0);
     if (e == cudaSuccess) e = cudaMemsetAsync(d.brick_owner, 0, sizeof(unsigned long long) * places, 0);
-    if (e == cudaSuccess) e = cudaMemsetAsync(d.brick_count, 0, sizeof(int32_t) * places, 0);
+    if (e == cudaSuccess) e = cudaMemsetAsync(d.brick_count, 0, sizeof(unsigned long long) * places, 0);
     if (e == cudaSuccess) e = cudaMemsetAsync(d.brick_cell, 0xff, sizeof(int32_t) * kBrickCells * places, 0);
     if (e == cudaSuccess) e = launch_reset(d, 0);
     if (e == cudaSuccess) e = cudaStreamSynchronize(0);
