@@ -919,11 +919,12 @@ int itm_mlp_loss_grad(const float *params_dev, const float *feat_dev, const floa
 {
     if (n <= 0 || !params_dev || !feat_dev || !labels_dev || !scratch_dev || !grad_dev || !loss_dev) return ITM_ERR_ARG;
     cudaStream_t st = (cudaStream_t)stream;
-    static const cudaError_t attr =
+    // on every call: the attribute belongs to the current device and is gone after its reset
+    const cudaError_t attr =
         cudaFuncSetAttribute(mlp_step_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(StepSmem));
     if (attr != cudaSuccess) return check_cuda(attr);
-    // one tile per CTA up to one CTA per SM; beyond that, CTAs take several
-    // tiles in turn, and their rows of partial sums stay few
+    // one tile per CTA while every CTA is resident at once; beyond that, CTAs
+    // take several tiles in turn, and their rows of partial sums stay few
     const int tiles = (n - 1) / kTS + 1;
     const int grid = std::min(tiles, step_grid());
     mlp_step_kernel<<<grid, kStepThreads, sizeof(StepSmem), st>>>(params_dev, feat_dev, labels_dev, n,
