@@ -476,7 +476,9 @@ cudaError_t launch_select(const SceneDev &s, const SwapDev &w, cudaStream_t st)
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int g = std::max(1, std::min(4 * sms, (s.nv + 255) / 256));
     swap_scan_kernel<OUT><<<g, 256, 0, st>>>(s, w);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     swap_count_kernel<OUT><<<n_chunks, kSelThreads, 0, st>>>(s, w);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     swap_select_kernel<OUT><<<n_chunks, kSelThreads, 0, st>>>(s, w, n_chunks);
     return cudaGetLastError();
 }
@@ -554,17 +556,21 @@ int itm_swap_out(itm_scene *sc, itm_stream stream)
     sc->last_stream = st;
     const SwapDev w = swap_dev(sc);
     cudaError_t e = recover(sc, st);
+    // the first launch that is refused ends the call: a later one would work on
+    // the header of a selection or a compaction that did not run
     if (e == cudaSuccess) e = launch_select<true>(sc->d, w, st);
     if (e != cudaSuccess) return check_cuda(e);
     if (sc->d.weight_mode == 0)
         swap_out_kernel<0><<<move_grid(w.k), kMoveThreads, 0, st>>>(sc->d, w);
     else
         swap_out_kernel<1><<<move_grid(w.k), kMoveThreads, 0, st>>>(sc->d, w);
+    if ((e = cudaGetLastError()) != cudaSuccess) return check_cuda(e);
     int dev = 0, sms = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int g = std::max(1, std::min(2 * sms, (sc->d.nv + 255) / 256));
     swap_compact_find_kernel<<<g, 256, 0, st>>>(sc->d, w);
+    if ((e = cudaGetLastError()) != cudaSuccess) return check_cuda(e);  // the blocks that moved stay in the prefix, unused
     swap_compact_pair_kernel<<<std::max(1, std::min(g, (w.k + 255) / 256)), 256, 0, st>>>(sc->d, w);
     return check_cuda(cudaGetLastError());
 }

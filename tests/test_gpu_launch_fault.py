@@ -267,3 +267,37 @@ for g, o in scenes:
     assert g.stats()["allocated_blocks"] == len(g.export(False)[0])
     assert same_volume(g, o)
 """ % (n, n))
+
+
+@pytest.mark.parametrize("n", range(1, 7))
+def test_swap_out(package, n):
+    """Each launch of a swap-out refused in turn (scan, count, select, move, the two of the compaction): up to the
+    move every block stays, after it those that moved are not found in device memory."""
+    run(package, r"""
+g, o = itm.Scene(**w.params), itm.Scene(**w.params)
+for s in (g, o):
+    s.swap_enable(1 << 14, 0)
+    for k in (0, 1, 2):
+        s.process(depth(k), ci, pose(k), *maps())
+refused(%d, g.swap_out)
+if %d > 4:
+    o.swap_out()
+for k in (9, 5, 0):
+    m = [maps(), maps()]
+    for s, x in ((g, m[0]), (o, m[1])):
+        s.raycast(ci, pose(0), *x)
+    assert same(*m), k
+    for s in (g, o):
+        s.allocate(depth(k), ci, pose(k))
+        s.swap_in()
+        s.integrate(depth(k), ci, pose(k))
+    assert same_volume(g, o), k
+assert g.status() == o.status() == 0
+for s in (g, o):
+    s.swap_out()
+    s.process(depth(3), ci, pose(3), *maps())
+m = [maps(), maps()]
+g.raycast(ci, pose(3), *m[0])
+o.raycast(ci, pose(3), *m[1])
+assert same(*m) and same_volume(g, o) and g.status() == o.status() == 0
+""" % (n, n))
