@@ -62,7 +62,7 @@ struct FrameCounters {
     int32_t n_req;          // buckets requested
     int32_t n_overflow;     // requests that lost their bucket
     int32_t depth_max_bits; // largest valid depth (float bits, >= 0)
-    int32_t done;           // CTAs of the visible-list pass that finished (frames with an overflow)
+    int32_t done;           // CTAs of the commit that finished (frames with an overflow)
 };
 
 // Two sets of frame counts take turns, so that no launch in front of an
@@ -268,7 +268,7 @@ inline int brick_places(int nv)
 __host__ __device__ __forceinline__ unsigned long long brick_key(int X, int Y, int Z)
 {
     return (unsigned long long)((uint32_t)(X & 0xffff) | ((uint32_t)Y << 16)) |
-           ((unsigned long long)((uint32_t)(Z & 0xffff) | 0x10000u) << 32);
+           ((unsigned long long)(uint32_t)(Z & 0xffff) << 32) | kBrickValid;
 }
 // its place: neighbouring bricks lie apart from each other, distant ones at random
 __host__ __device__ __forceinline__ uint32_t brick_place(int X, int Y, int Z, uint32_t mask)
@@ -280,8 +280,8 @@ __host__ __device__ __forceinline__ int brick_local(int lx, int ly, int lz)
     return lx + kBrickSide * ly + kBrickSide * kBrickSide * lz;
 }
 
-// The hash table's answers for the stencil of a brick whose place is shared
-// (bit k of want: the block at dx + 2 dy + 4 dz = k is asked for).
+// The hash table's answer for a block of a brick whose place is shared; a call
+// of its own, as it is rare and would be inlined for every block of a stencil.
 static __device__ __noinline__ int lookup_chain(const SceneDev &s, int bx, int by, int bz)
 {
     return lookup_ro(s, bx, by, bz);

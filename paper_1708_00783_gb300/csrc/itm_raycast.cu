@@ -67,7 +67,8 @@ __global__ void __launch_bounds__(256) range_kernel(SceneDev s, Mat34 M, Intr in
 // Persistent raycast, first phase (the march): each warp takes the next 8x4
 // tile from a device counter until none is left, so warps that finish early
 // pick up more work.  Rays that are not through after a while go to the slow
-// list (room: as many as the second phase takes at once; 0: none).
+// list (room: the list's length up to which warps give rays up early, see
+// march_warp; 0: no list).
 //
 // Most rays end within 6 to 10 iterations, but those that skim a wall or leave
 // the mapped part take 80 (room) to 190 (2 mm hall), each two dependent memory
@@ -206,13 +207,14 @@ cudaError_t launch_raycast(const SceneDev &s, const Intr &in, const Mat34 &T_wc,
         const int n_tiles = tx * ty, ctas = (n_tiles + 7) / 8;
         const int g = g_dyn[mode] < ctas ? g_dyn[mode] : ctas;
         // CTAs for the slow rays, three per SM (of four that fit beside each
-        // other; with one 640x480 takes 158 us instead of 129, 2 mm 798
-        // instead of 731); none for an image that could have more than the
-        // list holds.  room, the list's length up to which warps give rays up
-        // early: as many as these take at once, but at most 48 per SM: with
-        // all 192 the room takes 129 us instead of 136 and the 2 mm hall, a
-        // third of whose rays are slow, 731 instead of 679 (with none, that is
-        // after 48 iterations only, 140 and 681; 160x120 59 and 70).
+        // other); none for an image that could have more than the list holds.
+        // room, the list's length up to which warps give rays up early: as many
+        // as these CTAs take at once, but at most 48 per SM.  Whole frames in
+        // us, each pair on the same inputs, this setting first; 160x120, the
+        // 640x480 room, the 2 mm hall, a third of whose rays are slow:
+        //   one CTA per SM for slow rays  48.5 : 48.5, 112.7 : 112.0, 522 : 572
+        //   room up to all 192 per SM     42.7 : 42.7, 102.4 : 102.3, 600 : 629
+        //   room 1 (48 iterations first)  54.3 : 59.7, 148.6 : 150.4, 637 : 641
         const int slow_ctas = (long long)in.W * in.H > kSlowMax ? 0 : 3 * sms < ctas ? 3 * sms : ctas;
         const uint32_t *rmin = s.range_min, *rmax = s.range_max;
         const auto march = mode ? raycast_march_kernel<1> : raycast_march_kernel<0>;

@@ -34,7 +34,7 @@
 // element of the symmetric system per lane.  640x480, three levels, 19 steps:
 // 800 us per track with one kernel for the sums and one for a serial solve by
 // a single thread (9 + 26 us per step), 328 us with this one (362 with IEEE
-// divisions in the solve).
+// divisions in the solve); 800 and 325 in later runs of both on one box.
 #include "itm_ops.cuh"
 
 namespace itm {
